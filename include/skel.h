@@ -431,8 +431,7 @@ int skel_test_set_updown(skel_handle h, int code);
  * direction the launch shape of the up/down kernel (1, 2, 4 or 8 warps per
  * CTA sharing a 32-row block, with the blocks staged through registers or by
  * asynchronous copies; every shape adds the same partial sums in the same
- * order), the pipeline depth of the on-the-fly tensor-core kernel (4, 6
- * or 8 bulk-copy stages; same arithmetic), and for the tensor-core
+ * order), and for the tensor-core
  * translations (real kernels, nrhs >= 4) whether the
  * kernel values are evaluated on the fly or read from a store (the choice
  * between operators stored and evaluated on the fly: the per-tile and the
@@ -457,8 +456,8 @@ typedef struct {
     int    n_changed;         /* of those, choices unlike the default rule                      */
     double ms_updown_default; /* their summed time with the default rule                        */
     double ms_updown_tuned;   /* and with the chosen variants                                   */
-    int    tc_stages;         /* pipeline depth (bulk-copy stages) chosen for the on-the-fly
-                                 tensor-core kernel: 4, 6 or 8 (0: not tuned)                  */
+    int    tc_stages;         /* bulk-copy stages of the on-the-fly tensor-core kernel: 6
+                                 (0: not timed)                                                  */
     double ms_sym;            /* one tensor-core pass reading the symmetric store (-1: not timed) */
     int    tcs_stages;        /* form chosen for the per-tile stored kernel (store_stages: 4, 5
                                  or 8); 0: not tuned                                             */

@@ -40,6 +40,7 @@
 #include "device.h"
 #include "skel_kernels.cuh"
 #include "tc_kernels.cuh"
+#include "tc_near.cuh"
 #include "tc_complex.cuh"
 #include "tc_stored_ring.cuh"
 #include "tc_updown.cuh"
@@ -324,6 +325,8 @@ void permute(bool out, const DevicePlan* dp, const S* src, S* dst, int nrhs, cud
     }
 }
 
+constexpr int64_t kResidentGroups = 4 * 152;   // groups of the on-the-fly kernel that run at a time
+
 constexpr int kProfEvents = 8;   // 7 phase boundaries + the start of the main translation kernel
 constexpr int kMainEvent = 7;
 
@@ -363,16 +366,12 @@ NearArgs<Real, CPLX> near_args(DevicePlan* dp, DeviceBuffers* b, const WorkItem*
 void set_tc_attributes() {
     static bool done = false;
     if (done) return;
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecNone, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecNone, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecNone, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecNone, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecNone, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecNone, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecSym>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
-    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecSym>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecTiles>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<0, kRecSym>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
+    CUDA_CHECK(cudaFuncSetAttribute(tc_near_kernel<1, kRecSym>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmemRequest));
     CUDA_CHECK(cudaFuncSetAttribute(tc_stored_kernel<0, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, tcs_smem_request<4>()));
     CUDA_CHECK(cudaFuncSetAttribute(tc_stored_kernel<1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, tcs_smem_request<4>()));
     CUDA_CHECK(cudaFuncSetAttribute(tc_stored_kernel<0, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, tcs_smem_request<8>()));
@@ -399,6 +398,9 @@ int run_tc(DevicePlan* dp, DeviceBuffers* b, int nrhs, cudaStream_t st, int& tc_
     }
     TcArgs t;
     t.items = dp->tc_items;
+    t.units = (const TcUnit*)dp->tc_units;
+    t.part0 = dp->tc_part0;
+    t.parts = dp->tc_parts;
     t.tiles = dp->tc_tiles;
     t.X = (const float4*)b->X;
     t.Xlo = (const float4*)b->Xlo;
@@ -461,15 +463,14 @@ int run_tc(DevicePlan* dp, DeviceBuffers* b, int nrhs, cudaStream_t st, int& tc_
                               : tc_stored_kernel<1, 4><<<g, kTcThreads, tcs_smem_request<4>(), st>>>(t);
                 }
             } else {
-                // pipeline depth: the autotuner's choice (same arithmetic for every depth)
-                const unsigned g = (unsigned)dp->n_tc;
-                switch (dp->tc_stages) {
-                    case 4: kidx == 0 ? tc_near_kernel<0, kRecNone, 4><<<g, kTcThreads, kTcSmemRequest, st>>>(t)
-                                      : tc_near_kernel<1, kRecNone, 4><<<g, kTcThreads, kTcSmemRequest, st>>>(t); break;
-                    case 8: kidx == 0 ? tc_near_kernel<0, kRecNone, 8><<<g, kTcThreads, kTcSmemRequest, st>>>(t)
-                                      : tc_near_kernel<1, kRecNone, 8><<<g, kTcThreads, kTcSmemRequest, st>>>(t); break;
-                    default: kidx == 0 ? tc_near_kernel<0, kRecNone, 6><<<g, kTcThreads, kTcSmemRequest, st>>>(t)
-                                       : tc_near_kernel<1, kRecNone, 6><<<g, kTcThreads, kTcSmemRequest, st>>>(t); break;
+                if (t.withhold_item >= 0) t.withhold_item = dp->unit0_item;
+                kidx == 0 ? tc_near_kernel<0><<<(unsigned)dp->n_units, kNearThreads, kNearSmemRequest, st>>>(t)
+                          : tc_near_kernel<1><<<(unsigned)dp->n_units, kNearThreads, kNearSmemRequest, st>>>(t);
+                if (dp->n_split > 0) {
+                    CUDA_CHECK(cudaGetLastError());
+                    kidx == 0 ? tc_segments_kernel<0><<<(unsigned)dp->n_split, 256, 0, st>>>(t, dp->tc_split)
+                              : tc_segments_kernel<1><<<(unsigned)dp->n_split, 256, 0, st>>>(t, dp->tc_split);
+                    ++launches;
                 }
             }
             CUDA_CHECK(cudaGetLastError());
@@ -623,7 +624,12 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
     dp->store_mode = mode;
     dp->bytes += bytes;
     dp->stored_bytes = floats * (int64_t)sizeof(float);
+    TcUnit* units = nullptr;                               // one item per unit
     try {
+        std::vector<TcUnit> one((size_t)dp->n_tc);
+        for (size_t i = 0; i < one.size(); ++i) one[i] = TcUnit{(int32_t)i, -1, 0, 0, 0, (INT32_MAX / 2 / kTcGroup) * kTcGroup};
+        int64_t unit_bytes = 0;
+        units = upload(one, unit_bytes);
         DeviceBuffers* b = dp->p32;
         CUDA_CHECK(cudaMemsetAsync(b->Q, 0, (size_t)dp->n_tot * sizeof(float), st));
         set_tc_attributes();
@@ -633,6 +639,9 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
         CUDA_CHECK(cudaGetLastError());
         TcArgs t;
         t.items = dp->tc_items;
+        t.units = units;
+        t.part0 = nullptr;
+        t.parts = nullptr;
         t.tiles = dp->tc_tiles;
         t.X = (const float4*)b->X;
         t.Xlo = (const float4*)b->Xlo;
@@ -650,11 +659,11 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
         t.withhold_item = -1;
         const unsigned g = (unsigned)dp->n_tc;
         if (mode == 2) {
-            if (dp->kind == 0) tc_near_kernel<0, kRecSym><<<g, kTcThreads, kTcSmemRequest, st>>>(t);
-            else tc_near_kernel<1, kRecSym><<<g, kTcThreads, kTcSmemRequest, st>>>(t);
+            if (dp->kind == 0) tc_near_kernel<0, kRecSym><<<g, kNearThreads, kNearSmemRequest, st>>>(t);
+            else tc_near_kernel<1, kRecSym><<<g, kNearThreads, kNearSmemRequest, st>>>(t);
         } else {
-            if (dp->kind == 0) tc_near_kernel<0, kRecTiles><<<g, kTcThreads, kTcSmemRequest, st>>>(t);
-            else tc_near_kernel<1, kRecTiles><<<g, kTcThreads, kTcSmemRequest, st>>>(t);
+            if (dp->kind == 0) tc_near_kernel<0, kRecTiles><<<g, kNearThreads, kNearSmemRequest, st>>>(t);
+            else tc_near_kernel<1, kRecTiles><<<g, kNearThreads, kNearSmemRequest, st>>>(t);
         }
         CUDA_CHECK(cudaGetLastError());
         CUDA_CHECK(cudaStreamSynchronize(st));
@@ -662,11 +671,88 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
         CUDA_CHECK(cudaMemcpy(&stv, dp->status, sizeof(int), cudaMemcpyDeviceToHost));
         if (stv != 0) throw Error(-4, "the fill pass of the stored tiles timed out");
     } catch (...) {
+        cudaFree(units);
         drop_tiles(dp);
         throw;
     }
+    cudaFree(units);
 }
 
+
+// The on-the-fly kernel's units: two items with consecutive rows of one box
+// share a CTA and the tiles it copies; the other items pair up by the length
+// of their lists. Longest first. A plan with few tiles has its long lists cut
+// into parts of whole segments (kTcGroup tiles), so that the chip's 2 x 152
+// resident CTAs get work of about the same length; tc_segments_kernel adds
+// the segments of a cut item. Neither grouping nor cutting changes a result.
+struct Units {
+    std::vector<TcUnit> units;
+    std::vector<int64_t> part0;                            // per item (see TcArgs)
+    std::vector<int32_t> split;                            // the cut items
+    int64_t segments = 0;                                  // segments of the cut items
+};
+Units make_units(const std::vector<TcItem>& items) {
+    auto len = [&](int32_t i) { return items[i].list_hi - items[i].list_lo; };
+    int64_t tiles = 0;
+    for (size_t i = 0; i < items.size(); ++i) tiles += len((int32_t)i);
+    // a part: about a quarter of what each of the 608 groups gets in all
+    const int64_t share = tiles / (4 * kResidentGroups);
+    const int cut = (int)std::max<int64_t>(1, (share + kTcGroup / 2) / kTcGroup) * kTcGroup;
+    const bool small = share < kTcGroup * 4;
+    std::vector<int32_t> order(items.size());
+    for (size_t i = 0; i < items.size(); ++i) order[i] = (int32_t)i;
+    std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return items[x].row_off < items[y].row_off; });
+    std::vector<int32_t> mate(items.size(), -1);
+    for (size_t i = 0; i + 1 < order.size(); ++i) {
+        const TcItem &x = items[order[i]], &y = items[order[i + 1]];
+        if (x.box < 0 || x.box != y.box || x.nrows != kTcRows || y.row_off != x.row_off + kTcRows ||
+            len(order[i]) != len(order[i + 1]))
+            continue;
+        mate[order[i]] = order[i + 1];
+        mate[order[i + 1]] = -2;
+        ++i;
+    }
+    Units r;
+    r.part0.assign(items.size(), -1);
+    // (item or pair, first tile, tiles) pieces, longest first
+    struct Piece {
+        int32_t a, b, lo, n;
+    };
+    std::vector<Piece> pieces;
+    for (size_t i = 0; i < items.size(); ++i) {
+        if (mate[i] == -2) continue;
+        const int n = len((int32_t)i);
+        const bool split = small && n > cut;
+        const int step = split ? cut : std::max(n, 1);
+        for (int t = 0; t < std::max(n, 1); t += step)
+            pieces.push_back(Piece{(int32_t)i, mate[i], t, std::min(step, n - t)});
+        if (!split) continue;
+        for (int32_t it : {(int32_t)i, mate[i]}) {
+            if (it < 0) continue;
+            r.part0[it] = r.segments;
+            r.segments += (n + kTcGroup - 1) / kTcGroup;
+            r.split.push_back(it);
+        }
+    }
+    std::stable_sort(pieces.begin(), pieces.end(),
+                     [](const Piece& x, const Piece& y) { return length_class(x.n) > length_class(y.n); });
+    const int whole = (INT32_MAX / 2 / kTcGroup) * kTcGroup;
+    auto count = [&](const Piece& p) { return r.part0[p.a] >= 0 ? cut : whole; };
+    const Piece* single = nullptr;
+    for (const Piece& p : pieces) {
+        if (p.b >= 0) {
+            r.units.push_back(TcUnit{p.a, p.b, 1, p.lo, p.lo, count(p)});
+        } else if (!single || count(*single) != count(p)) {
+            if (single) r.units.push_back(TcUnit{single->a, -1, 0, single->lo, 0, count(*single)});
+            single = &p;
+        } else {
+            r.units.push_back(TcUnit{single->a, p.a, 0, single->lo, p.lo, count(p)});
+            single = nullptr;
+        }
+    }
+    if (single) r.units.push_back(TcUnit{single->a, -1, 0, single->lo, 0, count(*single)});
+    return r;
+}
 
 // The symmetric store of the stored-operator mode (tc_kernels.cuh): the row
 // chunks of every tensor-core item, and per (tile, row chunk) the stored
@@ -977,6 +1063,18 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
         dp->tc_tiles = upload(lay.tc_tiles, dp->bytes);
         dp->tc_items = upload(lay.tc_items, dp->bytes);
         dp->n_tc = (int64_t)lay.tc_items.size();
+        if (dp->n_tc > 0 && !dp->cplx) {
+            const Units u = make_units(lay.tc_items);
+            dp->n_units = (int64_t)u.units.size();
+            dp->unit0_item = u.units[0].a;
+            dp->tc_units = upload(u.units, dp->bytes);
+            dp->n_split = (int64_t)u.split.size();
+            if (dp->n_split > 0) {
+                dp->tc_part0 = upload(u.part0, dp->bytes);
+                dp->tc_split = upload(u.split, dp->bytes);
+                dp->tc_parts = dalloc<float>((size_t)u.segments * kTcRows * kTcN, dp->bytes);
+            }
+        }
         if (dp->n_tc > 0 && (!dp->cplx || dp->kind == 2)) {
             dp->chunk_start = upload(lay.chunk_start, dp->bytes);
             dp->chunk_cnt = upload(lay.chunk_cnt, dp->bytes);
@@ -1037,7 +1135,8 @@ void device_plan_destroy(DevicePlan* dp) {
     cudaSetDevice(dp->device);
     void* ptrs[] = {dp->box_off, dp->box_n, dp->box_nslot, dp->slot_start, dp->pos, dp->eop, dp->eop2, dp->up, dp->task_src, dp->task_mask, dp->task_flags, dp->items,
                     dp->part_ptr, dp->part_idx, dp->stage_in, dp->stage_out, dp->mix_items, dp->tc_tiles,
-                    dp->tc_items, dp->tc_part_ptr, dp->tc_part_idx, dp->status,
+                    dp->tc_items, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
+                    dp->tc_part_ptr, dp->tc_part_idx, dp->status,
                     dp->chunk_start, dp->chunk_cnt, dp->chunk_center, dp->tc_b, dp->tc_a, dp->tc_abase,
                     dp->tc_qmask, dp->tc_refs, dp->tc_isym, dp->ud_items_up, dp->ud_items_down,
                     dp->ud_a_up, dp->ud_a_down, dp->ud_tp, dp->ud_ttp, dp->ud_tp_off, dp->ud_ttp_off};
@@ -1175,16 +1274,8 @@ TuneReport device_autotune(DevicePlan* dp, int nrhs, bool allow_store, void* str
             auto tc = [&] { run_tc<float, false>(dp, b, nrhs, st, passes); };
             keep_a = dp->tc_a;
             dp->tc_a = nullptr;                            // time the on-the-fly kernel
-            // its pipeline depth (bulk-copy stages): the fastest of 4, 6, 8
-            rep.ms_onfly = 1e30;
-            int best_ns = kNS;
-            for (int ns : {4, 6, 8}) {
-                dp->tc_stages = ns;
-                const double ms = time_ms(tc, 3);
-                if (ms < rep.ms_onfly) rep.ms_onfly = ms, best_ns = ns;
-            }
-            dp->tc_stages = best_ns;
-            rep.tc_stages = best_ns;
+            rep.ms_onfly = time_ms(tc, 3);
+            rep.tc_stages = kNearPairs;
             dp->tc_a = keep_a;
             keep_a = nullptr;
             // the stores: the one the plan holds, and (allow_store) each one

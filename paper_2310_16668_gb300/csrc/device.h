@@ -45,6 +45,14 @@ struct DevicePlan {
     SrcTile* tc_tiles = nullptr;
     TcItem* tc_items = nullptr;
     int64_t n_tc = 0;
+    void* tc_units = nullptr;              // on-the-fly kernel: its CTAs' work (TcUnit)
+    int64_t n_units = 0;
+    int unit0_item = 0;                    // first item of the first unit (test hook)
+    // small plans: tile lists cut over several units, summed per segment
+    int64_t* tc_part0 = nullptr;           // per item: its first segment's sums (-1: not cut)
+    float* tc_parts = nullptr;
+    int32_t* tc_split = nullptr;           // the cut items
+    int64_t n_split = 0;
     int64_t tc_n_slots = 0;
     int64_t* tc_part_ptr = nullptr;        // per entry: its partial sums (tensor-core mode)
     int64_t* tc_part_idx = nullptr;
@@ -73,7 +81,6 @@ struct DevicePlan {
     // FP32 up/down launch shape per level: warps per CTA (0: the default
     // rule), set by the autotuner
     std::vector<int8_t> ud_warps_up, ud_warps_down;
-    int tc_stages = 6;                     // bulk-copy stages of the on-the-fly tensor-core kernel (4, 6, 8)
     int tcs_stages = 4;                    // stages per CTA of the per-tile stored kernel (4 or 8)
     // tensor-core upward / downward passes (FP32_TC, real kernels): per
     // direction the work items (UdItem) grouped by level and their A blobs

@@ -153,7 +153,7 @@ struct TcItem {                         // 64 bytes
     int32_t nslot;
     int32_t slot_start[kMaxSlots + 1];  // first row of each slot (may be < 0 for a box's later rows)
     int32_t list_lo, list_hi;           // its tiles: [list_lo, list_hi) of tc_tiles
-    int32_t slot;                       // unused (the item writes its rows of U directly)
+    int32_t box;                        // the box whose rows these are (-1: packed leaves)
 };
 static_assert(sizeof(TcItem) == 64, "TcItem layout");
 

@@ -335,7 +335,7 @@ void build_layout(const Plan& p, Layout& lay) {
         }
         // the whole list stays one item: its rows get exactly one writer
         it.list_hi = (int32_t)lay.tc_tiles.size();
-        it.slot = 0;
+        it.box = tg.size() == 1 && is_tc(tg[0].box) ? (int32_t)tg[0].box : -1;
         lay.tc_items.push_back(it);
     };
     for (int64_t b = 0; b < nb; ++b) {
@@ -455,6 +455,7 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
             it.row_off += e0[s];
             it.list_lo = (int32_t)(it.list_lo + t0[s]);
             it.list_hi = (int32_t)(it.list_hi + t0[s]);
+            if (it.box >= 0) it.box = (int32_t)(it.box + b0[s]);
             m.tc_items.push_back(it);
         }
         for (int64_t v : l.box_chunk0) m.box_chunk0.push_back(v < 0 ? -1 : v + c0[s]);

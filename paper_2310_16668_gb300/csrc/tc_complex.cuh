@@ -54,12 +54,6 @@ static_assert(sizeof(TcSharedC<kNSC>) <= kTccSmemRequest, "shared memory plan");
 
 __device__ __forceinline__ float2 tc_f2(float x) { return make_float2(x, x); }
 
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
-                    "r"(v[7]) : "memory");
-}
-
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
@@ -287,7 +281,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
             tmem_ld8(tbase + lane_off + kColD + 32u * (m & 1) + (uint32_t)(kColsC * quarter), v);
 #pragma unroll
             for (int c = 0; c < kColsC; ++c) acc[c] += __uint_as_float(v[c]);
-            if (m % kTcGroup == kTcGroup - 1) {
+            if (m % kTcOuter == kTcOuter - 1) {
 #pragma unroll
                 for (int c = 0; c < kColsC; ++c) {
                     S.outer[c][tid] += acc[c];

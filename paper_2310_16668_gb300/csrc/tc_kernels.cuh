@@ -60,9 +60,9 @@ constexpr int kTcCompute = 128 * kTpr;         // compute threads
 constexpr int kSrcPerThread = 32 / kTpr;       // sources of a tile each compute thread evaluates
 constexpr int kTcThreads = kTcCompute + 64;    // + the producer warp and the MMA warp
 constexpr int kTcN = 32;                       // right-hand sides per pass (MMA N)
-constexpr int kTcGroup = 128;                  // tiles summed in registers before the outer sum
-constexpr int kNS = 6;                         // data stages (bulk-copy destinations) by default;
-                                               // the autotuner may pick 4 or 8 (same arithmetic)
+constexpr int kTcGroup = 128;                  // tiles of a segment (summed in registers; segments add up in U)
+constexpr int kTcOuter = 128;                  // symmetric store, complex kernel: tiles summed in registers
+                                               // before the outer sum
 constexpr int kNA = 3;                         // A-operand buffers in tensor memory
 constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kColD = 0;                  // accumulators D0 [0,32), D1 [32,64)
@@ -71,32 +71,11 @@ constexpr uint32_t kSleepNs = 20000;           // suspend hint of one wait attem
 constexpr uint64_t kWaitLimitNs = 2000000000ull; // a wait gives up after 2 s (TcArgs::wait_ns)
 
 // one source chunk as the prep kernel lays it out in global memory and one
-// bulk copy moves it: B hi, B lo, source coordinates (hi, lo)
-constexpr int kChunkFloats = 2 * 1024 + 2 * 128;
-struct alignas(128) TcStage {
-    float bhi[32 * 32];                        // B operand, TF32 hi (bulk-copied, already converted)
-    float blo[32 * 32];                        // B operand, TF32 lo
-    float4 xh[32];                             // source coordinates (hi)
-    float4 xl[32];                             // lo parts (touching-leaf tiles)
-    SrcTile tile;                              // 64 B: the tile's descriptor (its own copy)
-};
-static_assert(offsetof(TcStage, tile) == kChunkFloats * 4, "chunk blob is contiguous in the stage");
-// per compute warp: for each target slot its 32 rows touch, the coordinates
-// of its kSrcPerThread sources, one array per axis (x, y, z); a source the
-// slot skips sits at kFar
-constexpr int kWarpSlotFloats = 3 * kSrcPerThread;
+// bulk copy moves it: B hi, B lo, then the 32 source coordinates as one array
+// per axis (x, y, z), hi parts then lo parts (a thread reads four sources of
+// an axis with one 16-byte load)
+constexpr int kChunkFloats = 2 * 1024 + 2 * 96;
 constexpr float kFar = 1e30f;                  // r^2 from here overflows to +inf: 1/r = 0
-template <int NS>
-struct TcShared {
-    TcStage st[NS];
-    float wc[kTcCompute / 32][kMaxSlots * kWarpSlotFloats];
-    float outer[kTcN / kTpr][kTcCompute];      // per compute thread: the sum of its flushed tile groups
-    uint64_t full[NS], afull[NS], empty[NS];   // per data stage
-    uint32_t tmem;
-    uint32_t slots;
-};
-constexpr int kTcSmemRequest = 112 * 1024;    // at most two CTAs (2 x 256 TMEM columns) per SM
-static_assert(sizeof(TcShared<8>) <= kTcSmemRequest, "shared memory plan");
 
 // Stored-operator mode (symmetric store). The rows of every tensor-core item
 // are whole source chunks ("row chunks", at most kMaxRc of them); the values
@@ -131,8 +110,21 @@ struct ItemSym {                               // 40 bytes per tensor-core item
 };
 static_assert(sizeof(ItemSym) == 40, "ItemSym layout");
 
+// A unit of the on-the-fly kernel (one CTA): two items, which share their
+// tiles if they hold consecutive rows of one box (equal tile lists), or parts
+// of items' tile lists
+struct TcUnit {
+    int32_t a, b;                              // items; b = -1: one item
+    int32_t shared;
+    int32_t lo_a, lo_b;                        // first tile of each item's list (a multiple of kTcGroup)
+    int32_t count;                             // tiles from there, at most (a multiple of kTcGroup)
+};
+
 struct TcArgs {
     const TcItem* items;
+    const TcUnit* units;                       // on-the-fly kernel: the CTAs' work
+    const int64_t* part0;                      // per item: its first segment in parts, -1 if it is not cut
+    float* parts;                              // sums of the segments of cut items, 128 rows x 32 (null: none)
     const SrcTile* tiles;                      // item i's tiles: [list_lo, list_hi) of this array
     const float4* X;
     const float4* Xlo;
@@ -234,11 +226,14 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void* src, uin
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
 }
 
-// B operand layout (K-major, no swizzle): core matrix = 8 right-hand sides x
-// 4 sources (16 bytes per row); the 4 groups of 8 right-hand sides of one
-// 4-source slab are contiguous (SBO = 128 B) and slabs follow along K
-// (LBO = 512 B): element (n, j) at byte (j/4)*512 + n*16 + (j%4)*4.
+// B operand layout (K-major, no swizzle): core matrix = 8 columns x 4 sources
+// (16 bytes per row); the groups of 8 columns of one 4-source slab are
+// contiguous (SBO = 128 B) and slabs follow along K (LBO). Real kernels: 64
+// columns per slab, the 32 right-hand sides' TF32 hi parts, then their lo
+// parts (LBO = 1 KB; the lo parts alone start 512 B on). Complex kernels: 32
+// columns per slab, hi and lo parts as separate 4 KB operands (LBO = 512 B).
 constexpr uint32_t kBLbo = 512, kBSbo = 128;
+constexpr uint32_t kBLboReal = 1024, kBLoPart = 512;
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
@@ -246,6 +241,21 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     d |= (uint64_t)((kBSbo >> 4) & 0x3FFF) << 32;   // SBO: next group of 8 rows (N)
     d |= (uint64_t)1 << 46;                          // descriptor version
     return d;                                        // base offset 0, no swizzle
+}
+
+// the low word of the descriptor of a real chunk's B operand at addr; per
+// K-step of 8 sources add kDescStep, for the lo columns add kDescLoPart
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) {
+    return ((addr >> 4) & 0x3FFF) | (((kBLboReal >> 4) & 0x3FFF) << 16);
+}
+constexpr uint32_t kDescHi = ((kBSbo >> 4) & 0x3FFF) | (1u << 14);   // SBO; descriptor version
+constexpr uint32_t kDescStep = 2u * kBLboReal / 16u, kDescLoPart = kBLoPart / 16u;
+
+// d (+)= A B^T; acc: accumulate (else overwrite d)
+__device__ __forceinline__ void mma_tf32_lo(uint32_t d, uint32_t a, uint32_t desc_lo, uint32_t idesc, bool acc) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 b;\n setp.ne.b32 p, %5, 0;\n mov.b64 b, {%2, %3};\n"
+                 " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], b, %4, p;\n}\n"
+                 :: "r"(d), "r"(a), "r"(desc_lo), "r"(kDescHi), "r"(idesc), "r"((uint32_t)acc));
 }
 
 __device__ __forceinline__ void mma_tf32(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
@@ -258,28 +268,23 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
                  :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
                     "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]),
-                    "r"(v[15]) : "memory");
+                    "r"(v[15]));
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                   "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
-                   "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
-                   "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                 : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]),
+                    "r"(v[7]));
 }
 
+// (the wait is part of the statement: the values are not used before it)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+                 " tcgen05.wait::ld.sync.aligned;"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
                    "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
                    "=r"(v[15])
                  : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // kernel value without its constant factor (see Green<>). 3D: the PTX
@@ -297,56 +302,10 @@ template <int KIND, bool ADJ> __device__ __forceinline__ float tc_green(float r2
     return (!ADJ || r2 > 1.17549435e-38f) ? y : 0.f;
 }
 
-// 16 sources (j0 .. j0+15) against this thread's target, two sources per
-// paired FP32 instruction. c: this row's slot copy of these 16 coordinates
-// (axes AX floats apart); xl: the stage's lo parts (touching-leaf tiles);
-// nt / nl: the negated target coordinates.
-template <int KIND, bool ADJ, int AX>
-__device__ __forceinline__ void tc_eval16(const float* c, const float4* xl, int j0, float4 nt, float4 nl,
-                                          uint32_t* ghi, uint32_t* glo) {
-    const float2 ntx = make_float2(nt.x, nt.x), nty = make_float2(nt.y, nt.y), ntz = make_float2(nt.z, nt.z);
-    float2 nlx, nly, nlz;
-    if (ADJ) nlx = make_float2(nl.x, nl.x), nly = make_float2(nl.y, nl.y), nlz = make_float2(nl.z, nl.z);
-    const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        // four sources per axis in one 16-byte load
-        const float4 X = *reinterpret_cast<const float4*>(&c[4 * q]);
-        const float4 Y = *reinterpret_cast<const float4*>(&c[AX + 4 * q]);
-        const float4 Z = *reinterpret_cast<const float4*>(&c[2 * AX + 4 * q]);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int jj = 4 * q + 2 * h;
-            float2 dx = __fadd2_rn(h ? make_float2(X.z, X.w) : make_float2(X.x, X.y), ntx);
-            float2 dy = __fadd2_rn(h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y), nty);
-            float2 dz = __fadd2_rn(h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y), ntz);
-            if (ADJ) {
-                const float4 l0 = xl[j0 + jj], l1 = xl[j0 + jj + 1];
-                dx = __fadd2_rn(dx, __fadd2_rn(make_float2(l0.x, l1.x), nlx));
-                dy = __fadd2_rn(dy, __fadd2_rn(make_float2(l0.y, l1.y), nly));
-                dz = __fadd2_rn(dz, __fadd2_rn(make_float2(l0.z, l1.z), nlz));
-            }
-            float2 r2 = __fmul2_rn(dx, dx);
-            r2 = __ffma2_rn(dy, dy, r2);
-            r2 = __ffma2_rn(dz, dz, r2);
-            const float2 g = make_float2(tc_green<KIND, ADJ>(r2.x), tc_green<KIND, ADJ>(r2.y));
-            // Veltkamp's split: hi = t - (t - g) with t = (2^13 + 1) g keeps 11
-            // significant bits of g (exactly a TF32 value, rounded to
-            // nearest); lo = g - hi is exact
-            const float2 t = __fmul2_rn(g, split);
-            const float2 hi = __ffma2_rn(__ffma2_rn(g, m1, t), m1, t);
-            const float2 lo = __ffma2_rn(hi, m1, g);
-            ghi[jj] = __float_as_uint(hi.x);
-            ghi[jj + 1] = __float_as_uint(hi.y);
-            glo[jj] = __float_as_uint(lo.x);
-            glo[jj + 1] = __float_as_uint(lo.y);
-        }
-    }
-}
-
 // One source chunk for right-hand sides r0 .. r0+31, laid out as the stage
 // holds it: the B operand in the shared-memory layout of the MMA (element
-// (n, j) at float (j/4)*128 + n*4 + j%4), split into TF32 hi (rounded to
+// (n, j) at float (j/4)*256 + n*4 + j%4, its lo part 128 floats on; complex:
+// (j/4)*128, the lo parts 1024 floats on), split into TF32 hi (rounded to
 // nearest) and lo = q - hi, then the chunk's 32 source coordinates (hi part
 // minus the box centre: FP32 then resolves them to the box size, not to the
 // domain size) and their lo parts; entries past the chunk and columns past
@@ -394,8 +353,13 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
         h.z = __uint_as_float(to_tf32(x[2]));
         h.w = __uint_as_float(to_tf32(x[3]));
         l = make_float4(x[0] - h.x, x[1] - h.y, x[2] - h.z, x[3] - h.w);
-        *reinterpret_cast<float4*>(blob + 2048 * part + jq * 128 + n * 4) = h;
-        *reinterpret_cast<float4*>(blob + 2048 * part + 1024 + jq * 128 + n * 4) = l;
+        if constexpr (CPLX) {
+            *reinterpret_cast<float4*>(blob + 2048 * part + jq * 128 + n * 4) = h;
+            *reinterpret_cast<float4*>(blob + 2048 * part + 1024 + jq * 128 + n * 4) = l;
+        } else {
+            *reinterpret_cast<float4*>(blob + jq * 256 + n * 4) = h;
+            *reinterpret_cast<float4*>(blob + jq * 256 + 128 + n * 4) = l;
+        }
     }
     // the chunk's coordinates: hi parts measured from the box centre, then
     // the lo parts (zero past cnt)
@@ -409,8 +373,46 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
             } else {
                 c = Xlo[start + j];
             }
+        } else if (!CPLX && threadIdx.x < 32) {
+            c = make_float4(kFar, kFar, kFar, 0.f);
         }
-        reinterpret_cast<float4*>(blob + kXoff)[threadIdx.x] = c;
+        if constexpr (CPLX) {
+            reinterpret_cast<float4*>(blob + kXoff)[threadIdx.x] = c;
+        } else {
+            float* d = blob + kXoff + (threadIdx.x >> 5) * 96 + j;
+            d[0] = c.x;
+            d[32] = c.y;
+            d[64] = c.z;
+        }
+    }
+}
+
+// U[row][r0 + c0 ..] = scale * v (the first segment of an item) or += it: a
+// row has one writer, so its segments add up in order
+template <int KIND, int NC>
+__device__ __forceinline__ void tc_add_rows(const TcArgs& a, int64_t row, int c0, bool add, const float* v) {
+    const float scale = (float)green_scale<KIND>();
+    float* u = a.U + row * a.nrhs + a.r0 + c0;
+    const int left = a.nrhs - a.r0 - c0;
+    if (a.nrhs % 4 == 0 && left >= NC) {
+        float4* u4 = reinterpret_cast<float4*>(u);
+#pragma unroll
+        for (int c = 0; c < NC / 4; ++c) {
+            float4 w = make_float4(__fmul_rn(scale, v[4 * c]), __fmul_rn(scale, v[4 * c + 1]),
+                                   __fmul_rn(scale, v[4 * c + 2]), __fmul_rn(scale, v[4 * c + 3]));
+            if (add) {
+                const float4 o = u4[c];
+                w = make_float4(__fadd_rn(o.x, w.x), __fadd_rn(o.y, w.y), __fadd_rn(o.z, w.z), __fadd_rn(o.w, w.w));
+            }
+            u4[c] = w;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < left) {
+                const float w = __fmul_rn(scale, v[c]);
+                u[c] = add ? __fadd_rn(u[c], w) : w;
+            }
     }
 }
 
@@ -424,258 +426,6 @@ constexpr int kTileFloats = 128 * 32;          // the largest tile
 // float4 index of (row, quad) in a tile with quad mask qm
 __device__ __forceinline__ int tile_word(uint32_t qm, int quad, int row, int nrows) {
     return __popc(qm & ((1u << quad) - 1u)) * nrows + row;
-}
-
-// REC: the fill pass of a stored-operator mode also writes the kernel values
-// it evaluates to a.A: kRecTiles every tile's values as the MMA consumes them
-// (hi + lo, masked), kRecSym the blocks this tile records for the symmetric
-// store (every source of the chunk, unmasked).
-constexpr int kRecNone = 0, kRecTiles = 1, kRecSym = 2;
-template <int KIND, int REC = kRecNone, int NS = kNS>
-__global__ void __launch_bounds__(kTcThreads, 2) tc_near_kernel(const TcArgs a) {
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    TcShared<NS>& S = *reinterpret_cast<TcShared<NS>*>(smem_raw);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const TcItem* itp = a.items + blockIdx.x;
-    const int64_t row_off = itp->row_off;
-    const int nrows = itp->nrows, nslot = itp->nslot, list_lo = itp->list_lo;
-    const int ntile = itp->list_hi - list_lo;
-
-    if (tid == 0) {
-        S.slots = 0;
-        for (int s = 0; s < NS; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_addr(&S.full[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(sm_addr(&S.afull[s])), "r"(kTcCompute));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_addr(&S.empty[s])));
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(sm_addr(&S.tmem)), "r"(kTmemCols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tbase = S.tmem;
-    bool err = false;
-
-    if (warp == kTcCompute / 32) {
-        // ---------------- producer warp: bulk copies up to NS tiles ahead ----------------
-        // the lanes fetch the descriptors of 32 tiles at a time; lane 0
-        // issues each tile's copies
-        for (int t0 = 0; t0 < ntile; t0 += 32) {
-            const int d_chunk = t0 + lane < ntile ? a.tiles[list_lo + t0 + lane].chunk : 0;
-            const int nb = min(32, ntile - t0);
-            for (int i = 0; i < nb; ++i) {
-                const int t = t0 + i;
-                const int s = t % NS;
-                const int chunk = __shfl_sync(0xffffffffu, d_chunk, i);
-                if (t >= NS && !mbar_wait(sm_addr(&S.empty[s]), (uint32_t)(((t - NS) / NS) & 1), a.wait_ns)) err = true;
-                const bool hold = t == 0 && (int)blockIdx.x == a.withhold_item;
-                if (hold && !withhold_first_tile(sm_addr(&S.afull[0]), a.wait_ns)) err = true;
-                if (lane == 0) {
-                    // two bulk copies: the chunk (B hi, B lo, coordinates) and
-                    // the tile's descriptor
-                    const uint32_t bar = sm_addr(&S.full[s]);
-                    mbar_arrive_tx(bar, 4u * kChunkFloats + 64u);
-                    bulk_g2s_hint(sm_addr(S.st[s].bhi), a.B + (int64_t)chunk * kChunkFloats, 4u * kChunkFloats, bar,
-                                  l2_evict_last());
-                    bulk_g2s_hint(sm_addr(&S.st[s].tile), a.tiles + list_lo + t, 64u, bar, l2_evict_first());
-                    if (hold && !mbar_wait(bar, 0u, a.wait_ns)) err = true;
-                }
-                __syncwarp();
-            }
-        }
-        if (lane == 0) {
-            // all bulk copies have landed before the CTA may exit
-            for (int t = (ntile > NS ? ntile - NS : 0); t < ntile; ++t)
-                if (!mbar_wait(sm_addr(&S.full[t % NS]), (uint32_t)((t / NS) & 1), a.wait_ns)) err = true;
-        }
-    } else if (warp == kTcCompute / 32 + 1) {
-        // ---------------- MMA issuer (one thread) ----------------
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
-                                   ((128u >> 4) << 24);
-            for (int m = 0; m < ntile; ++m) {
-                const int s = m % NS, ab = m % kNA;
-                if (!mbar_wait(sm_addr(&S.afull[s]), (uint32_t)((m / NS) & 1), a.wait_ns)) err = true;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t bh = sm_addr(S.st[s].bhi), bl = sm_addr(S.st[s].blo);
-                const uint32_t d = tbase + kColD + 32u * (m & 1);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t ahi = tbase + kColA + 64u * ab + 8u * k, alo = ahi + 32u;
-                    mma_tf32(d, ahi, smem_desc(bh + 2u * kBLbo * k), idesc, k > 0 ? 1u : 0u);
-                    mma_tf32(d, ahi, smem_desc(bl + 2u * kBLbo * k), idesc, 1u);
-                    mma_tf32(d, alo, smem_desc(bh + 2u * kBLbo * k), idesc, 1u);
-                }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             :: "r"(sm_addr(&S.empty[s])) : "memory");
-            }
-        }
-    } else {
-        // ---------------- compute warps ----------------
-        const int row = tid & 127, half = tid >> 7;
-        const bool valid = row < nrows;
-        int myslot = 0;
-        for (int c = 1; c < nslot; ++c)
-            if (row >= itp->slot_start[c]) myslot = c;
-        float4 tx = make_float4(0.f, 0.f, 0.f, 0.f), tl = tx;
-        if (valid) {
-            tx = a.X[row_off + row];
-            tl = a.Xlo[row_off + row];
-        }
-        const float4 nl = make_float4(-tl.x, -tl.y, -tl.z, 0.f);
-        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-        // the slots this warp's 32 rows fall in: s_lo .. s_lo + nsw - 1
-        const int r_first = 32 * (warp & 3), r_last = min(r_first + 31, nrows - 1);
-        int s_lo = 0, s_hi = 0;
-        for (int c = 1; c < nslot; ++c) {
-            if (r_first >= itp->slot_start[c]) s_lo = c;
-            if (r_last >= itp->slot_start[c]) s_hi = c;
-        }
-        const int nsw = max(1, s_hi - s_lo + 1);
-        const int myloc = min(max(myslot - s_lo, 0), kMaxSlots - 1);
-        float* wc = S.wc[warp];
-        constexpr int kCols = kTcN / kTpr;                     // accumulator columns this thread owns
-        constexpr uint32_t kKeepMask = kSrcPerThread == 32 ? 0xFFFFFFFFu : (1u << kSrcPerThread) - 1u;
-        const int j0 = kSrcPerThread * half;
-        int64_t tfill = 0;                                     // per-tile fill: floats of the tiles before
-        // fill pass: this row's row chunk and its row in it
-        int rk = 0, rl = row, rm = 1;
-        int64_t rref0 = 0;
-        if constexpr (REC == kRecSym) {
-            const ItemSym* is = a.isym + blockIdx.x;
-            rm = is->m;
-            rref0 = is->ref0;
-            for (int k = 1; k < rm; ++k)
-                if (row >= is->ro[k]) rk = k;
-            rl = row - is->ro[rk];
-        }
-        // two-level FP32 sum: acc adds the tiles of a group of kTcGroup, the
-        // shared-memory `outer` adds the groups (keeps long lists accurate)
-        float acc[kCols];
-#pragma unroll
-        for (int c = 0; c < kCols; ++c) {
-            acc[c] = 0.f;
-            S.outer[c][tid] = 0.f;
-        }
-        auto drain = [&](int m) {                              // add tile m's accumulator
-            if (!mbar_wait(sm_addr(&S.empty[m % NS]), (uint32_t)((m / NS) & 1), a.wait_ns)) err = true;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t v[kCols];
-            const uint32_t col = tbase + lane_off + kColD + 32u * (m & 1) + (uint32_t)(kCols * half);
-            if constexpr (kCols == 32) tmem_ld32(col, v);
-            else tmem_ld16(col, v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-            if (m % kTcGroup == kTcGroup - 1) {
-#pragma unroll
-                for (int c = 0; c < kCols; ++c) {
-                    S.outer[c][tid] += acc[c];
-                    acc[c] = 0.f;
-                }
-            }
-        };
-        for (int u = 0; u < ntile; ++u) {
-            const int s = u % NS;
-            if (!mbar_wait(sm_addr(&S.full[s]), (uint32_t)((u / NS) & 1), a.wait_ns)) err = true;
-            TcStage& st = S.st[s];
-            const bool adj = (st.tile.flags & TASK_ADJ) != 0;
-            // the target measured from the source box's centre (the frame of
-            // the chunk's coordinates); touching leaves keep hi and lo apart
-            const float cx = st.tile.cen[0], cy = st.tile.cen[1], cz = st.tile.cen[2];
-            const float4 nt = adj ? make_float4(cx - tx.x, cy - tx.y, cz - tx.z, 0.f)
-                                  : make_float4((cx - tx.x) - tl.x, (cy - tx.y) - tl.y, (cz - tx.z) - tl.z, 0.f);
-            const uint32_t keep = valid ? (st.tile.keep[myslot] >> j0) & kKeepMask : 0u;
-            // this warp's copy of its sources per slot and axis; a skipped
-            // source (and any j >= cnt, never kept) sits at kFar. Every lane
-            // has finished reading the previous tile's copy.
-            __syncwarp();
-            for (int p = lane; p < nsw * kSrcPerThread; p += 32) {
-                const int ls = p / kSrcPerThread, jj = p % kSrcPerThread;
-                const float4 v = st.xh[j0 + jj];
-                // (the fill pass records every source of the chunk, unmasked:
-                // each reader of a stored block applies its own keep mask)
-                const bool kept = REC == kRecSym ? (j0 + jj < st.tile.cnt)
-                                                 : ((st.tile.keep[s_lo + ls] >> (j0 + jj)) & 1u) != 0u;
-                float* d = wc + ls * kWarpSlotFloats + jj;
-                d[0] = kept ? v.x : kFar;
-                d[kSrcPerThread] = kept ? v.y : kFar;
-                d[2 * kSrcPerThread] = kept ? v.z : kFar;
-            }
-            __syncwarp();
-            if (u >= 2) drain(u - 2);                          // frees accumulator (u & 1)
-            // A buffer u % kNA was last read by MMA(u - kNA), complete since drain(u - 2)
-            const uint32_t acol = tbase + lane_off + kColA + 64u * (u % kNA) + (uint32_t)j0;
-            const float* c = wc + myloc * kWarpSlotFloats;
-            const bool none = REC != kRecSym && __all_sync(0xffffffffu, keep == 0);
-#pragma unroll
-            for (int g = 0; g < kSrcPerThread / 16; ++g) {
-                uint32_t ghi[16], glo[16];
-                if (none) {
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) ghi[jj] = glo[jj] = 0u;
-                } else if (adj) {
-                    tc_eval16<KIND, true, kSrcPerThread>(c + 16 * g, st.xl, j0 + 16 * g, nt, nl, ghi, glo);
-                } else {
-                    tc_eval16<KIND, false, kSrcPerThread>(c + 16 * g, st.xl, j0 + 16 * g, nt, nl, ghi, glo);
-                }
-                tmem_st16(acol + 16u * g, ghi);
-                tmem_st16(acol + 32u + 16u * g, glo);
-                if constexpr (REC == kRecTiles) {
-                    const uint32_t qm = a.qmask[list_lo + u];
-                    float4* dst = reinterpret_cast<float4*>(a.A + a.abase[blockIdx.x] + tfill);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int jj = 4 * q, quad = 4 * half + q;
-                        if (valid && ((qm >> quad) & 1u)) dst[tile_word(qm, quad, row, nrows)] =
-                            make_float4(__uint_as_float(ghi[jj]) + __uint_as_float(glo[jj]),
-                                        __uint_as_float(ghi[jj + 1]) + __uint_as_float(glo[jj + 1]),
-                                        __uint_as_float(ghi[jj + 2]) + __uint_as_float(glo[jj + 2]),
-                                        __uint_as_float(ghi[jj + 3]) + __uint_as_float(glo[jj + 3]));
-                    }
-                    tfill += (int64_t)__popc(qm) * nrows * 4;
-                }
-                if constexpr (REC == kRecSym) {
-                    // this row's block of the tile, if this tile records it
-                    // (stored as this row chunk x the tile's chunk)
-                    const BlockRef rf = a.refs[rref0 + (int64_t)u * rm + rk];
-                    if (valid && (rf.flags & kRefRecord)) {
-                        const int jb = j0 + 16 * g;
-#pragma unroll
-                        for (int jj = 0; jj < 16; ++jj)
-                            if (jb + jj < st.tile.cnt)
-                                a.A[rf.off + (int64_t)(jb + jj) * rf.pitch + rl] =
-                                    __uint_as_float(ghi[jj]) + __uint_as_float(glo[jj]);
-                    }
-                }
-            }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(sm_addr(&S.afull[s]));
-        }
-        for (int m = (ntile >= 2 ? ntile - 2 : 0); m < ntile; ++m) drain(m);
-#pragma unroll
-        for (int c = 0; c < kCols; ++c) acc[c] += S.outer[c][tid];
-        if (valid) {
-            const float scale = (float)green_scale<KIND>();
-            const int64_t base = (row_off + row) * a.nrhs;
-            const int c0 = a.r0 + kCols * half;
-#pragma unroll
-            for (int c = 0; c < kCols; ++c)
-                if (c0 + c < a.nrhs) a.U[base + c0 + c] = scale * acc[c];
-        }
-    }
-    if (err) atomicExch(a.status, 1);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tbase), "r"(kTmemCols));
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -693,16 +443,61 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_near_kernel(const TcArgs a) 
 // tc_near_kernel, so both give the same result bit for bit. Bound: HBM,
 // nrows x 128 bytes of kernel values per tile.
 static_assert(kSrcPerThread == 16, "stored tiles assume two compute threads per row");
-// Four stages in flight need the shared memory that tc_near_kernel gives to
-// the outer sums, so here they live in tensor memory, where two A buffers
-// leave room: D0, D1 [0, 64), A[b] hi at 64 + 64 b, lo at 96 + 64 b (b < 2),
-// the outer sums at [192, 224). Two A buffers suffice: the buffer of tile u
-// was last read by MMA(u - 2), which drain(u - 2) has waited for before tile
-// u is written.
+// Tensor memory: D0, D1 [0, 64) for the pairs in turn, L [64, 96), A[b] hi at
+// 128 + 64 b, lo at 160 + 64 b (b < 2). Two A buffers suffice: the buffer of
+// tile u was last read by MMA(u - 2), which has been waited for before tile u
+// is written.
 // NST data stages (24 KB each): 4 with two CTAs per SM, or 8 with one CTA
 // per SM (the autotuner times both).
 constexpr int kNAS = 2;                        // A buffers
-constexpr uint32_t kColOuter = 192;
+constexpr uint32_t kColSL = 64, kColSA = 128;
+
+// The stored kernels' MMAs of tile m (its B operand at bh): the sum of
+// tc_near.cuh, with pair p's hi*hi products in D[p % 2]
+__device__ __forceinline__ void tcs_mma_tile(uint32_t tbase, int m, uint32_t bh, uint32_t idesc) {
+    const uint32_t d = tbase + kColD + 32u * ((uint32_t)(m >> 1) & 1u), l = tbase + kColSL;
+    const uint32_t ahi = tbase + kColSA + 64u * (uint32_t)(m % kNAS), alo = ahi + 32u, b0 = smem_desc_lo(bh);
+    const bool first = !(m & 1), seg = (m & (kTcGroup - 1)) == 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t dbh = b0 + kDescStep * k, dbl = dbh + kDescLoPart;
+        mma_tf32_lo(l, ahi + 8u * k, dbl, idesc, !seg || k > 0);
+        mma_tf32_lo(l, alo + 8u * k, dbh, idesc, true);
+        mma_tf32_lo(d, ahi + 8u * k, dbh, idesc, !first || k > 0);
+    }
+}
+
+// The stored kernels' register sums of one thread (16 columns from tcol of
+// its lane): a pair's D is added when the pair after the next starts, before
+// the MMAs that restart it
+struct TcSums {
+    float2 acc[8];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ void add(uint32_t taddr) {
+        uint32_t v[16];
+        tmem_ld16(taddr, v);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            acc[c] = __fadd2_rn(acc[c], make_float2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1])));
+    }
+    // pair p of the segment (its MMAs are done)
+    __device__ __forceinline__ void pair(uint32_t tcol, int p) { add(tcol + kColD + 32u * ((uint32_t)p & 1u)); }
+    // the segment's value: the pairs not yet added, then L
+    __device__ __forceinline__ void finish(uint32_t tcol, int len, float* v) {
+        const int np = (len + 1) / 2;
+        for (int p = max(np - 2, 0); p < np; ++p) pair(tcol, p);
+        if (np > 0) add(tcol + kColSL);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            v[2 * c] = acc[c].x;
+            v[2 * c + 1] = acc[c].y;
+        }
+        clear();
+    }
+};
 struct alignas(128) TcTileStage {
     float b[2 * 1024];                         // B hi, B lo (the first 8 KB of the chunk block)
     float4 ga[kTileFloats / 4];                // the tile's kept quads
@@ -790,18 +585,10 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
             const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
                                    ((128u >> 4) << 24);
             for (int m = 0; m < ntile; ++m) {
-                const int s = m % NST, ab = m % kNAS;
+                const int s = m % NST;
                 if (!mbar_wait(sm_addr(&S.afull[s]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t bh = sm_addr(S.st[s].b), bl = bh + 4u * 1024u;
-                const uint32_t d = tbase + kColD + 32u * (m & 1);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t ahi = tbase + kColA + 64u * ab + 8u * k, alo = ahi + 32u;
-                    mma_tf32(d, ahi, smem_desc(bh + 2u * kBLbo * k), idesc, k > 0 ? 1u : 0u);
-                    mma_tf32(d, ahi, smem_desc(bl + 2u * kBLbo * k), idesc, 1u);
-                    mma_tf32(d, alo, smem_desc(bh + 2u * kBLbo * k), idesc, 1u);
-                }
+                tcs_mma_tile(tbase, m, sm_addr(S.st[s].b), idesc);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.empty[s])) : "memory");
             }
@@ -813,38 +600,21 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         constexpr int kCols = kTcN / kTpr;
         const int j0 = kSrcPerThread * half;
-        float acc[kCols];
-        const uint32_t ocol = tbase + lane_off + kColOuter + (uint32_t)(kCols * half);
-        {
-            uint32_t z[kCols];
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) {
-                acc[c] = 0.f;
-                z[c] = 0u;
-            }
-            tmem_st16(ocol, z);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        }
-        // the outer sums: this thread's 16 columns of lane `row`
-        auto flush = [&]() {
-            uint32_t v[kCols];
-            tmem_ld16(ocol, v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) {
-                v[c] = __float_as_uint(__uint_as_float(v[c]) + acc[c]);
-                acc[c] = 0.f;
-            }
-            tmem_st16(ocol, v);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        };
-        auto drain = [&](int m) {
+        const uint32_t tcol = tbase + lane_off + (uint32_t)(kCols * half);
+        TcSums sums;
+        sums.clear();
+        // wait for tile m's MMAs
+        auto done = [&](int m) {
             if (!mbar_wait(sm_addr(&S.empty[m % NST]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t v[kCols];
-            tmem_ld16(tbase + lane_off + kColD + 32u * (m & 1) + (uint32_t)(kCols * half), v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-            if (m % kTcGroup == kTcGroup - 1) flush();
+        };
+        // the segment that ends before tile u goes to U
+        auto flush = [&](int u) {
+            if (u > 0) done(u - 1);
+            const int s0 = u > 0 ? (u - 1) & ~(kTcGroup - 1) : 0;
+            float v[kCols];
+            sums.finish(tcol, u - s0, v);
+            if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
         };
         const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
         for (int u = 0; u < ntile; ++u) {
@@ -872,29 +642,21 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
                     glo[jj + 1] = __float_as_uint(lo.y);
                 }
             }
-            if (u >= 2) drain(u - 2);
-            const uint32_t acol = tbase + lane_off + kColA + 64u * (u % kNAS) + (uint32_t)j0;
+            if (u > 0 && (u & (kTcGroup - 1)) == 0) {
+                flush(u);
+            } else {
+                if (u >= 2) done(u - 2);
+                // before the pair that starts with tile u, the pair two before it
+                if (!(u & 1) && (u & (kTcGroup - 1)) >= 4) sums.pair(tcol, ((u & (kTcGroup - 1)) >> 1) - 2);
+            }
+            const uint32_t acol = tbase + lane_off + kColSA + 64u * (u % kNAS) + (uint32_t)j0;
             tmem_st16(acol, ghi);
             tmem_st16(acol + 32u, glo);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(sm_addr(&S.afull[s]));
         }
-        for (int m = (ntile >= 2 ? ntile - 2 : 0); m < ntile; ++m) drain(m);
-        {
-            uint32_t v[kCols];
-            tmem_ld16(ocol, v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-        }
-        if (valid) {
-            const float scale = (float)green_scale<KIND>();
-            const int64_t base = (row_off + row) * a.nrhs;
-            const int c0 = a.r0 + kCols * half;
-#pragma unroll
-            for (int c = 0; c < kCols; ++c)
-                if (c0 + c < a.nrhs) a.U[base + c0 + c] = scale * acc[c];
-        }
+        flush(ntile);
     }
     if (err) atomicExch(a.status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1066,14 +828,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_sym_kernel(const TcArgs a) {
                 const int s = mm % kNSY, ab = mm % kNA;
                 if (!mbar_wait(sm_addr(&S.afull[s]), (uint32_t)((mm / kNSY) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t bh = sm_addr(S.st[s].b), bl = bh + 4u * 1024u;
+                const uint32_t b0 = smem_desc_lo(sm_addr(S.st[s].b));
                 const uint32_t d = tbase + kColD + 32u * (mm & 1);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const uint32_t ahi = tbase + kColA + 64u * ab + 8u * k, alo = ahi + 32u;
-                    mma_tf32(d, ahi, smem_desc(bh + 2u * kBLbo * k), idesc, k > 0 ? 1u : 0u);
-                    mma_tf32(d, ahi, smem_desc(bl + 2u * kBLbo * k), idesc, 1u);
-                    mma_tf32(d, alo, smem_desc(bh + 2u * kBLbo * k), idesc, 1u);
+                    const uint32_t dbh = b0 + kDescStep * k, dbl = dbh + kDescLoPart;
+                    mma_tf32_lo(d, ahi, dbh, idesc, k > 0);
+                    mma_tf32_lo(d, ahi, dbl, idesc, true);
+                    mma_tf32_lo(d, alo, dbh, idesc, true);
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.empty[s])) : "memory");
@@ -1107,7 +870,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_sym_kernel(const TcArgs a) {
             tmem_ld16(tbase + lane_off + kColD + 32u * (mm & 1) + (uint32_t)(kCols * half), v);
 #pragma unroll
             for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-            if (mm % kTcGroup == kTcGroup - 1) {
+            if (mm % kTcOuter == kTcOuter - 1) {
 #pragma unroll
                 for (int c = 0; c < kCols; ++c) {
                     S.outer[c][tid] += acc[c];

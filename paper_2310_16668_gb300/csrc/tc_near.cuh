@@ -1,0 +1,542 @@
+// On-the-fly tensor-core translations (FP32_TC, real kernels): the kernel
+// values are evaluated by the CTA that multiplies them.
+//
+// A CTA owns a unit: two items with consecutive rows of one box (up to 256
+// rows, equal tile lists), or one item (up to 128 rows). It has four compute
+// warps, thread = row of each item, a producer warp that streams pairs of
+// tiles (chunks and descriptors) by bulk copies NS / 2 stages deep, and an
+// MMA warp. Between two hand-overs to the tensor core a thread evaluates 32
+// values: of two items, 16 sources for its row of each (the coordinates are
+// read once for both); of one item, one tile's 32 sources for its row. What a
+// hand-over costs (mbarrier waits, fences, tensor-memory waits: about as long
+// as 50 values' evaluation) is thus shared by 32 values a thread, and while
+// the tensor core works on one half of A the other half is written.
+//
+// The sum, the same for both forms and for the stored kernels (so all give
+// the same bits): an item's tile list is cut into segments of kTcGroup tiles
+// and a segment into pairs of tiles. The hi*hi products of a pair accumulate in
+// tensor memory (D: 8 K-steps) and are then added to an FP32 register sum;
+// the hi*lo and lo*hi products of the whole segment accumulate in a second
+// accumulator (L), which is 2^-11 of the first in size, so that its rounding
+// does not show, and is added at the segment's end. Segments are scaled and
+// added in order. Of the products of a tile only four MMAs thus round at the
+// size of the result (twelve did when all went into one accumulator), and a
+// pair needs one read of D. B holds hi and lo as 64 columns, so hi*hi and
+// hi*lo are one MMA into the adjacent columns of D and L: two MMAs per K-step
+// (an issuing thread needs 48 cycles for an MMA of 32 or of 64 columns).
+//
+// Masks: a tile's keep word of the row's slot. A row that keeps none of 8
+// sources sits at kFar (the kernel value is 0 there); where some row keeps a
+// part of the 8, values are selected one by one. Chunks shorter than 32
+// sources carry kFar coordinates past their end. A warp whose rows keep
+// nothing of a tile writes zeros, once; a warp without valid rows takes no
+// part.
+#pragma once
+
+#include <type_traits>
+
+#include "tc_kernels.cuh"
+
+namespace skel {
+
+constexpr int kNearCompute = 256;              // compute threads: two groups of 128 rows
+constexpr int kNearThreads = kNearCompute + 128;  // + two producer and two MMA warps
+// Registers: 384 threads x 2 CTAs launch with 80 each; the compute warpgroups
+// take what the last one gives up (256 x 104 + 128 x 32 = 384 x 80)
+constexpr int kNearRegsCompute = 104, kNearRegsOther = 32;
+static_assert(kNearCompute * kNearRegsCompute + 128 * kNearRegsOther <= kNearThreads * 80, "register split");
+// a group's tensor memory (128 columns): D, L, then A in two halves of 16
+// sources (hi 16 columns, lo 16 columns)
+constexpr uint32_t kColNearA = 64;
+constexpr int kNearPairs = 6;                  // stages of two tiles
+struct alignas(128) TcPairStage {
+    float chunk[2][kChunkFloats];              // B hi and lo, coordinates (hi, lo) of two tiles
+    SrcTile tile[2];
+};
+struct TcNearShared {
+    TcPairStage st[kNearPairs];
+    uint64_t full[kNearPairs], empty[kNearPairs];  // per stage: copies landed; MMAs of its readers done
+    uint64_t afull[2][2], done[2][2];          // per group and half of A: written; its MMAs done
+    uint32_t tmem;
+};
+constexpr int kNearSmemRequest = 113 * 1024;   // two CTAs (2 x 256 TMEM columns) per SM
+static_assert(sizeof(TcNearShared) <= kNearSmemRequest, "shared memory plan");
+
+// 8 sources (coordinates at x: 32 floats per axis; lo parts 96 floats on)
+// against this thread's target, two sources per paired FP32 instruction: the
+// kernel values in g, not masked. nt, nl: the negated target.
+template <int KIND, bool ADJ>
+__device__ __forceinline__ void tc_eval8(const float* x, float4 nt, float4 nl, float* g) {
+    constexpr int AX = 32, LO = 96;
+    const float2 ntx = make_float2(nt.x, nt.x), nty = make_float2(nt.y, nt.y), ntz = make_float2(nt.z, nt.z);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float4 X = *reinterpret_cast<const float4*>(x + 4 * q);
+        const float4 Y = *reinterpret_cast<const float4*>(x + AX + 4 * q);
+        float4 Z, LX, LY, LZ;
+        if (KIND != 0) Z = *reinterpret_cast<const float4*>(x + 2 * AX + 4 * q);
+        if (ADJ) {
+            LX = *reinterpret_cast<const float4*>(x + LO + 4 * q);
+            LY = *reinterpret_cast<const float4*>(x + LO + AX + 4 * q);
+            if (KIND != 0) LZ = *reinterpret_cast<const float4*>(x + LO + 2 * AX + 4 * q);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float2 dx = __fadd2_rn(h ? make_float2(X.z, X.w) : make_float2(X.x, X.y), ntx);
+            float2 dy = __fadd2_rn(h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y), nty);
+            if (ADJ) {
+                dx = __fadd2_rn(dx, __fadd2_rn(h ? make_float2(LX.z, LX.w) : make_float2(LX.x, LX.y),
+                                               make_float2(nl.x, nl.x)));
+                dy = __fadd2_rn(dy, __fadd2_rn(h ? make_float2(LY.z, LY.w) : make_float2(LY.x, LY.y),
+                                               make_float2(nl.y, nl.y)));
+            }
+            float2 r2 = __fmul2_rn(dx, dx);
+            r2 = __ffma2_rn(dy, dy, r2);
+            if (KIND != 0) {
+                float2 dz = __fadd2_rn(h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y), ntz);
+                if (ADJ)
+                    dz = __fadd2_rn(dz, __fadd2_rn(h ? make_float2(LZ.z, LZ.w) : make_float2(LZ.x, LZ.y),
+                                                   make_float2(nl.z, nl.z)));
+                r2 = __ffma2_rn(dz, dz, r2);
+            }
+            g[4 * q + 2 * h] = tc_green<KIND, ADJ>(r2.x);
+            g[4 * q + 2 * h + 1] = tc_green<KIND, ADJ>(r2.y);
+        }
+    }
+}
+
+// Veltkamp's split of 8 values into TF32 hi and lo: hi = t - (t - g) with
+// t = (2^13 + 1) g keeps 11 significant bits of g (a TF32 value, rounded to
+// nearest); lo = g - hi is exact. hi goes to the 8 tensor-memory columns from
+// taddr, lo to those 16 columns on.
+__device__ __forceinline__ void tc_split_store(const float* g, uint32_t taddr) {
+    const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+        const float2 v = make_float2(g[j], g[j + 1]);
+        const float2 t = __fmul2_rn(v, split);
+        const float2 h = __ffma2_rn(__ffma2_rn(v, m1, t), m1, t);
+        const float2 l = __ffma2_rn(h, m1, v);
+        hi[j] = __float_as_uint(h.x);
+        hi[j + 1] = __float_as_uint(h.y);
+        lo[j] = __float_as_uint(l.x);
+        lo[j + 1] = __float_as_uint(l.y);
+    }
+    tmem_st8(taddr, hi);
+    tmem_st8(taddr + 16u, lo);
+}
+
+// a[0..15] += the 32 tensor-memory columns from taddr of this thread's lane
+__device__ __forceinline__ void tmem_add32(uint32_t taddr, float2* a) {
+    uint32_t v[32];
+    tmem_ld16(taddr, v);
+    tmem_ld16(taddr + 16u, v + 16);
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+        a[c] = __fadd2_rn(a[c], make_float2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1])));
+}
+
+template <int N>
+__device__ __forceinline__ void tmem_zero(uint32_t taddr) {
+    uint32_t z[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) z[c] = 0u;
+#pragma unroll
+    for (int c = 0; c < N; c += 8) tmem_st8(taddr + c, z);
+}
+
+// REC: the fill pass of a stored-operator mode also writes the kernel values
+// it evaluates to a.A: kRecTiles every tile's values as the MMA consumes them
+// (masked), kRecSym the blocks this tile records for the symmetric store
+// (every source of the chunk, unmasked). Fill passes run one item per unit.
+constexpr int kRecNone = 0, kRecTiles = 1, kRecSym = 2;
+
+// one thread's targets and masks for a tile
+struct TcNearRow {
+    float4 x, lo;                              // coordinates (hi, lo)
+    int slot;                                  // its slot of the item
+    bool valid;
+};
+struct TcNearTile {
+    float4 nt, nl;                             // negated target: in the frame of the chunk; lo parts
+    uint32_t kw;                               // kept sources
+    bool none, some;                           // warp: no row keeps any source; some row keeps a part
+};
+template <int REC>
+__device__ __forceinline__ TcNearTile tc_near_tile(const TcNearRow& r, const SrcTile& st, uint32_t all, bool adj) {
+    TcNearTile t;
+    t.kw = r.valid ? st.keep[r.slot] : 0u;
+    t.none = REC == kRecNone && __all_sync(0xffffffffu, t.kw == 0u);
+    t.some = REC != kRecSym && __any_sync(0xffffffffu, t.kw != 0u && t.kw != all);
+    // the target measured from the source box's centre (the frame of the
+    // chunk's coordinates); touching leaves keep hi and lo apart
+    const float cx = st.cen[0], cy = st.cen[1], cz = st.cen[2];
+    t.nt = adj ? make_float4(cx - r.x.x, cy - r.x.y, cz - r.x.z, 0.f)
+               : make_float4((cx - r.x.x) - r.lo.x, (cy - r.x.y) - r.lo.y, (cz - r.x.z) - r.lo.z, 0.f);
+    t.nl = make_float4(-r.lo.x, -r.lo.y, -r.lo.z, 0.f);
+    if (REC != kRecSym && t.kw == 0u) t.nt.x = kFar;
+    return t;
+}
+// masks of 8 sources q: this row's target moved to kFar if it keeps none of
+// them; true if some row of the warp keeps a part of them
+__device__ __forceinline__ bool tc_near_cut(const TcNearTile& t, uint32_t all, int q, float4& at) {
+    at = t.nt;
+    if (!t.some) return false;
+    const uint32_t kb = t.kw >> (8 * q) & 0xFFu;
+    if (kb == 0u) at.x = kFar;
+    return __any_sync(0xffffffffu, kb != 0u && kb != (all >> (8 * q) & 0xFFu));
+}
+__device__ __forceinline__ void tc_near_select(const TcNearTile& t, int q, float* g) {
+    const uint32_t kb = t.kw >> (8 * q);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) g[j] = (kb >> j) & 1u ? g[j] : 0.f;
+}
+
+// The compute warps of one group: thread = row of the group's item.
+// st, full: the group's ring of NP stages; afull, done: its two halves of A;
+// tcol: its columns of tensor memory (D, L, A).
+template <int KIND, int REC>
+__device__ __forceinline__ bool tc_near_rows(const TcArgs& a, const TcPairStage* ring, const uint64_t* full, int np,
+                                             uint64_t* afull, const uint64_t* done, int item, int t_lo, int t_hi, float* parts,
+                                             int rot, uint32_t tcol) {
+    const int warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const TcItem* itp = a.items + item;
+    const int nrows = itp->nrows, list_lo = itp->list_lo;
+    // warp w always runs on scheduler w % 4: the 32-row blocks are dealt to the
+    // warps from a position that moves with the CTA
+    const int blk = (warp + rot) & 3, row = 32 * blk + lane;
+    if (32 * blk >= nrows) return true;
+    const uint32_t dcol = tcol + ((uint32_t)(warp * 32) << 16), acol = dcol + kColNearA;
+    TcNearRow rw;
+    rw.valid = row < nrows;
+    const int64_t urow = itp->row_off + row;
+    rw.slot = 0;
+    for (int c = 1; c < itp->nslot; ++c)
+        if (row >= itp->slot_start[c]) rw.slot = c;
+    rw.x = rw.lo = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rw.valid) {
+        rw.x = a.X[urow];
+        rw.lo = a.Xlo[urow];
+    }
+    // fill passes: this row's row chunk and its row in it; the floats of the
+    // tiles before the current one
+    int rk = 0, rl = row, rm = 1;
+    int64_t rref0 = 0, tfill = 0;
+    if constexpr (REC == kRecSym) {
+        const ItemSym* is = a.isym + item;
+        rm = is->m;
+        rref0 = is->ref0;
+        for (int k = 1; k < rm; ++k)
+            if (row >= is->ro[k]) rk = k;
+        rl = row - is->ro[rk];
+    }
+    bool ok = true;
+    uint32_t cnt = 0u;                                     // tiles handed over: the phases of afull and done
+    // half b of A is free: the previous tile's MMAs on it are done
+    auto wait_done = [&](int b) {
+        if (cnt > 0u) ok &= mbar_wait(sm_addr(&done[b]), (cnt - 1u) & 1u, a.wait_ns);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    auto hand_over = [&](int b) {
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sm_addr(&afull[b]));
+    };
+    float2 acc[16];
+    bool azero = false;                                    // A holds zeros in this warp's rows
+    int s = 0;
+    uint32_t ph = 0u;
+    int s0 = t_lo;
+    do {                                                   // segments (an item without tiles writes zeros)
+        const int send = min(s0 + kTcGroup, t_hi);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) acc[c] = make_float2(0.f, 0.f);
+        tmem_zero<64>(dcol);                               // D and L
+        for (int t = s0; t < send; ++t) {
+            const int ti = t & 1;
+            const TcPairStage& st = ring[s];
+            if (ti == 0) ok &= mbar_wait(sm_addr(&full[s]), ph, a.wait_ns);
+            const SrcTile& tl = st.tile[ti];
+            const float* xs = st.chunk[ti] + 2048;
+            const bool adj = (tl.flags & TASK_ADJ) != 0;
+            const uint32_t all = tl.cnt >= 32 ? 0xFFFFFFFFu : (1u << (tl.cnt & 31)) - 1u;
+            const TcNearTile ta = tc_near_tile<REC>(rw, tl, all, adj);
+            // before the first MMAs of a pair: the pair before it
+            auto drain = [&]() {
+                if (ti == 0 && t > s0) {
+                    wait_done(1);
+                    tmem_add32(dcol, acc);
+                    tmem_zero<32>(dcol);
+                }
+            };
+            if (ta.none) {
+                wait_done(0);
+                if (!azero) tmem_zero<32>(acol);
+                drain();
+                hand_over(0);
+                wait_done(1);
+                if (!azero) tmem_zero<32>(acol + 32u);
+                hand_over(1);
+                azero = true;
+            } else {
+                azero = false;
+                // CUT: some row keeps a part of the sources
+                auto tile = [&](auto ADJ, auto CUT) {
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const int q = 2 * b + e;
+                            float g[8];
+                            float4 at = ta.nt;
+                            bool cut = false;
+                            if constexpr (decltype(CUT)::value) cut = tc_near_cut(ta, all, q, at);
+                            tc_eval8<KIND, decltype(ADJ)::value>(xs + 8 * q, at, ta.nl, g);
+                            if constexpr (REC == kRecSym) {
+                                // this row's block of the tile, if this tile records it
+                                // (stored as this row chunk x the tile's chunk)
+                                const BlockRef rf = a.refs[rref0 + (int64_t)t * rm + rk];
+                                if (rw.valid && (rf.flags & kRefRecord)) {
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j)
+                                        if (8 * q + j < tl.cnt)
+                                            a.A[rf.off + (int64_t)(8 * q + j) * rf.pitch + rl] = g[j];
+                                }
+                            }
+                            if (cut) tc_near_select(ta, q, g);
+                            if constexpr (REC == kRecTiles) {
+                                const uint32_t qm = a.qmask[list_lo + t];
+                                float4* dst = reinterpret_cast<float4*>(a.A + a.abase[item] + tfill);
+#pragma unroll
+                                for (int h = 0; h < 2; ++h)
+                                    if (rw.valid && ((qm >> (2 * q + h)) & 1u))
+                                        dst[tile_word(qm, 2 * q + h, row, nrows)] =
+                                            make_float4(g[4 * h], g[4 * h + 1], g[4 * h + 2], g[4 * h + 3]);
+                            }
+                            if (e == 0) {
+                                wait_done(b);
+                                __syncwarp();
+                            }
+                            tc_split_store(g, acol + 32u * b + 8u * e);
+                        }
+                        if (b == 0) drain();
+                        hand_over(b);
+                    }
+                };
+                if (ta.some) {
+                    if (adj) tile(std::true_type{}, std::true_type{});
+                    else tile(std::false_type{}, std::true_type{});
+                } else {
+                    if (adj) tile(std::true_type{}, std::false_type{});
+                    else tile(std::false_type{}, std::false_type{});
+                }
+                if constexpr (REC == kRecTiles) tfill += (int64_t)__popc((uint32_t)a.qmask[list_lo + t]) * nrows * 4;
+            }
+            ++cnt;
+            if ((ti == 1 || t == send - 1) && ++s == np) s = 0, ph ^= 1u;
+        }
+        if (send > s0) {
+            // the last pair, then the segment's small products
+            wait_done(0);
+            wait_done(1);
+            tmem_add32(dcol, acc);
+            tmem_add32(dcol + 32u, acc);
+        }
+        if (rw.valid) {
+            float v[32];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) v[2 * c] = acc[c].x, v[2 * c + 1] = acc[c].y;
+            if (parts == nullptr) {
+                tc_add_rows<KIND, 32>(a, urow, 0, s0 > 0, v);
+            } else {
+                // a part of the item: its segments go to their own rows
+                float4* d = reinterpret_cast<float4*>(parts + ((int64_t)(s0 / kTcGroup) * kTcRows + row) * kTcN);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) d[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+            }
+        }
+        s0 += kTcGroup;
+    } while (s0 < t_hi);
+    return ok;
+}
+
+template <int KIND, int REC = kRecNone>
+__global__ void __launch_bounds__(kNearThreads, 2) tc_near_kernel(const TcArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    TcNearShared& S = *reinterpret_cast<TcNearShared*>(smem_raw);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const TcUnit un = a.units[blockIdx.x];
+    // one stream of tiles for both groups, or one each
+    const int np = un.shared ? kNearPairs : kNearPairs / 2;
+    // the tiles of group g's item this unit covers
+    auto tiles_lo = [&](int g) { return g ? un.lo_b : un.lo_a; };
+    auto tiles_hi = [&](int g) {
+        const TcItem& it = a.items[g ? un.b : un.a];
+        return min(tiles_lo(g) + un.count, it.list_hi - it.list_lo);
+    };
+
+    if (tid == 0) {
+        for (int s = 0; s < kNearPairs; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_addr(&S.full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;"
+                         :: "r"(sm_addr(&S.empty[s])), "r"(un.shared ? 2 : 1));
+        }
+        for (int g = 0; g < 2; ++g) {
+            // the warps that hold rows of the group's item (the others take no part)
+            const int warps = g == 1 && un.b < 0 ? 1 : (a.items[g ? un.b : un.a].nrows + 31) / 32;
+            for (int b = 0; b < 2; ++b) {
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(sm_addr(&S.afull[g][b])), "r"(warps));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(sm_addr(&S.done[g][b])));
+            }
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(sm_addr(&S.tmem)), "r"(kTmemCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tbase = S.tmem;
+    bool err = false;
+
+    if (warp >= kNearCompute / 32) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kNearRegsOther));
+        const int role = warp - kNearCompute / 32;           // 0, 1: producers; 2, 3: MMA issuers of the groups
+        const int g = role & 1;
+        const int item = g ? un.b : un.a;
+        const int ring = un.shared ? 0 : g * (kNearPairs / 2);
+        if (role < 2 && item >= 0 && !(g == 1 && un.shared)) {
+            // ---------------- producer: bulk copies up to np pairs ahead ----------------
+            const int list_lo = a.items[item].list_lo + tiles_lo(g), ntile = tiles_hi(g) - tiles_lo(g);
+            const bool hold = item == a.withhold_item;
+            const int npair = (ntile + 1) / 2;
+            int s = 0;
+            uint32_t ph = 1u;                                // phase of empty: passes at once in the first round
+            for (int p0 = 0; p0 < npair; p0 += 16) {
+                const int my_chunk = 2 * p0 + lane < ntile ? a.tiles[list_lo + 2 * p0 + lane].chunk : 0;
+                const int n = min(16, npair - p0);
+                for (int i = 0; i < n; ++i) {
+                    const int p = p0 + i;
+                    const int c0 = __shfl_sync(0xffffffffu, my_chunk, 2 * i);
+                    const int c1 = __shfl_sync(0xffffffffu, my_chunk, 2 * i + 1);
+                    const bool two = 2 * p + 1 < ntile;
+                    if (p >= np && !mbar_wait(sm_addr(&S.empty[ring + s]), ph, a.wait_ns)) err = true;
+                    if (hold && p == 0 && !withhold_first_tile(sm_addr(&S.afull[g][0]), a.wait_ns)) err = true;
+                    if (lane == 0) {
+                        TcPairStage& st = S.st[ring + s];
+                        const uint32_t bar = sm_addr(&S.full[ring + s]);
+                        const uint64_t keep = l2_evict_last();
+                        mbar_arrive_tx(bar, (two ? 2u : 1u) * (4u * kChunkFloats + 64u));
+                        bulk_g2s_hint(sm_addr(st.chunk[0]), a.B + (int64_t)c0 * kChunkFloats, 4u * kChunkFloats, bar, keep);
+                        if (two)
+                            bulk_g2s_hint(sm_addr(st.chunk[1]), a.B + (int64_t)c1 * kChunkFloats, 4u * kChunkFloats, bar,
+                                          keep);
+                        bulk_g2s_hint(sm_addr(st.tile), a.tiles + list_lo + 2 * p, two ? 128u : 64u, bar,
+                                      l2_evict_first());
+                        // (after a withheld tile the compute warps may run ahead of
+                        // the copies: each stage lands before it is armed again)
+                        if (hold && !mbar_wait(bar, ph ^ 1u, a.wait_ns)) err = true;
+                    }
+                    __syncwarp();
+                    if (++s == np) s = 0, ph ^= 1u;
+                }
+            }
+            if (lane == 0) {
+                // all bulk copies have landed and all commits have arrived
+                // before the CTA may exit
+                for (int p = max(npair - np, 0); p < npair; ++p) {
+                    if (!mbar_wait(sm_addr(&S.full[ring + p % np]), (uint32_t)((p / np) & 1), a.wait_ns)) err = true;
+                    if (!mbar_wait(sm_addr(&S.empty[ring + p % np]), (uint32_t)((p / np) & 1), a.wait_ns)) err = true;
+                }
+            }
+        } else if (role >= 2 && item >= 0) {
+            // ---------------- MMA issuer (one thread) ----------------
+            if (lane == 0) {
+                const int ntile = tiles_hi(g) - tiles_lo(g);
+                const uint32_t idesc32 =
+                    (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) | ((128u >> 4) << 24);
+                const uint32_t idesc64 =
+                    (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(2 * kTcN >> 3) << 17) | ((128u >> 4) << 24);
+                auto commit = [&](uint64_t* bar) {
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 :: "r"(sm_addr(bar)) : "memory");
+                };
+                const uint32_t dcol = tbase + 128u * g, acol = dcol + kColNearA;
+                int s = 0;
+                for (int t = 0; t < ntile; ++t) {
+                    const uint32_t b0 = smem_desc_lo(sm_addr(S.st[ring + s].chunk[t & 1]));
+                    const bool last = (t & 1) || t == ntile - 1;   // of its pair
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        if (!mbar_wait(sm_addr(&S.afull[g][b]), (uint32_t)t & 1u, a.wait_ns)) err = true;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            // D, L += hi [hi | lo]; L += lo hi
+                            const uint32_t desc = b0 + kDescStep * (2 * b + k), ac = acol + 32u * b + 8u * k;
+                            mma_tf32_lo(dcol, ac, desc, idesc64, true);
+                            mma_tf32_lo(dcol + 32u, ac + 16u, desc, idesc32, true);
+                        }
+                        if (b == 1 && last) commit(&S.empty[ring + s]);
+                        commit(&S.done[g][b]);
+                    }
+                    if (last && ++s == np) s = 0;
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kNearRegsCompute));
+        const int g = warp >> 2;
+        const int item = g ? un.b : un.a;
+        const int ring = un.shared ? 0 : g * (kNearPairs / 2);
+        float* parts = nullptr;
+        if (a.parts != nullptr && item >= 0 && a.part0[item] >= 0) parts = a.parts + a.part0[item] * (kTcRows * kTcN);
+        if (item >= 0 && !tc_near_rows<KIND, REC>(a, S.st + ring, S.full + ring, np, S.afull[g], S.done[g], item,
+                                                  tiles_lo(g), tiles_hi(g), parts,
+                                                  (int)(blockIdx.x + 2u * (uint32_t)g), tbase + 128u * g))
+            err = true;
+    }
+    if (err) atomicExch(a.status, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tbase), "r"(kTmemCols));
+    }
+}
+
+// The items whose lists were cut over several units: U = the sum of their
+// segments, in order (one CTA per item; a thread owns 4 columns of a row).
+// The scaling and the order of the additions are those of tc_add_rows.
+template <int KIND>
+__global__ void __launch_bounds__(256) tc_segments_kernel(const TcArgs a, const int32_t* __restrict__ split) {
+    const int item = split[blockIdx.x];
+    const TcItem it = a.items[item];
+    const int nseg = (it.list_hi - it.list_lo + kTcGroup - 1) / kTcGroup;
+    const float scale = (float)green_scale<KIND>();
+    const float* parts = a.parts + a.part0[item] * (kTcRows * kTcN);
+    for (int i = threadIdx.x; i < it.nrows * (kTcN / 4); i += 256) {
+        const int row = i / (kTcN / 4), c0 = 4 * (i % (kTcN / 4));
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int s = 0; s < nseg; ++s) {
+            const float4 v = *reinterpret_cast<const float4*>(parts + ((int64_t)s * kTcRows + row) * kTcN + c0);
+            const float4 w = make_float4(__fmul_rn(scale, v.x), __fmul_rn(scale, v.y), __fmul_rn(scale, v.z),
+                                         __fmul_rn(scale, v.w));
+            u = s == 0 ? w : make_float4(__fadd_rn(u.x, w.x), __fadd_rn(u.y, w.y), __fadd_rn(u.z, w.z),
+                                         __fadd_rn(u.w, w.w));
+        }
+        float* d = a.U + (it.row_off + row) * a.nrhs + a.r0 + c0;
+        const float* uv = &u.x;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (a.r0 + c0 + c < a.nrhs) d[c] = uv[c];
+    }
+}
+
+}  // namespace skel

@@ -119,19 +119,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
             const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
                                    ((128u >> 4) << 24);
             for (int m = 0; m < ntile; ++m) {
-                const int sa = m % NA, sb = m % NB, ab = m % kNAS;
+                const int sa = m % NA, sb = m % NB;
                 if (!mbar_wait(sm_addr(&S.afull[sa]), (uint32_t)((m / NA) & 1), a.wait_ns)) err = true;
                 if (!mbar_wait(sm_addr(&S.fullB[sb]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t bh = sm_addr(S.bb[sb].b), bl = bh + 4u * 1024u;
-                const uint32_t d = tbase + kColD + 32u * (m & 1);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t ahi = tbase + kColA + 64u * ab + 8u * k, alo = ahi + 32u;
-                    mma_tf32(d, ahi, smem_desc(bh + 2u * kBLbo * k), idesc, k > 0 ? 1u : 0u);
-                    mma_tf32(d, ahi, smem_desc(bl + 2u * kBLbo * k), idesc, 1u);
-                    mma_tf32(d, alo, smem_desc(bh + 2u * kBLbo * k), idesc, 1u);
-                }
+                tcs_mma_tile(tbase, m, sm_addr(S.bb[sb].b), idesc);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.emptyB[sb])) : "memory");
             }
@@ -143,38 +135,21 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         constexpr int kCols = kTcN / kTpr;
         const int j0 = kSrcPerThread * half;
-        float acc[kCols];
-        const uint32_t ocol = tbase + lane_off + kColOuter + (uint32_t)(kCols * half);
-        {
-            uint32_t z[kCols];
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) {
-                acc[c] = 0.f;
-                z[c] = 0u;
-            }
-            tmem_st16(ocol, z);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        }
-        auto flush = [&]() {
-            uint32_t v[kCols];
-            tmem_ld16(ocol, v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) {
-                v[c] = __float_as_uint(__uint_as_float(v[c]) + acc[c]);
-                acc[c] = 0.f;
-            }
-            tmem_st16(ocol, v);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        };
-        // tile m's MMAs are done once its B slot's commit phase has completed
-        auto drain = [&](int m) {
+        const uint32_t tcol = tbase + lane_off + (uint32_t)(kCols * half);
+        TcSums sums;
+        sums.clear();
+        // wait for tile m's MMAs
+        auto done = [&](int m) {
             if (!mbar_wait(sm_addr(&S.emptyB[m % NB]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            uint32_t v[kCols];
-            tmem_ld16(tbase + lane_off + kColD + 32u * (m & 1) + (uint32_t)(kCols * half), v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-            if (m % kTcGroup == kTcGroup - 1) flush();
+        };
+        // the segment that ends before tile u goes to U
+        auto flush = [&](int u) {
+            if (u > 0) done(u - 1);
+            const int s0 = u > 0 ? (u - 1) & ~(kTcGroup - 1) : 0;
+            float v[kCols];
+            sums.finish(tcol, u - s0, v);
+            if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
         };
         const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
         for (int u = 0; u < ntile; ++u) {
@@ -206,29 +181,21 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
                     glo[jj + 1] = __float_as_uint(lo.y);
                 }
             }
-            if (u >= 2) drain(u - 2);
-            const uint32_t acol = tbase + lane_off + kColA + 64u * (u % kNAS) + (uint32_t)j0;
+            if (u > 0 && (u & (kTcGroup - 1)) == 0) {
+                flush(u);
+            } else {
+                if (u >= 2) done(u - 2);
+                // before the pair that starts with tile u, the pair two before it
+                if (!(u & 1) && (u & (kTcGroup - 1)) >= 4) sums.pair(tcol, ((u & (kTcGroup - 1)) >> 1) - 2);
+            }
+            const uint32_t acol = tbase + lane_off + kColSA + 64u * (u % kNAS) + (uint32_t)j0;
             tmem_st16(acol, ghi);
             tmem_st16(acol + 32u, glo);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(sm_addr(&S.afull[sa]));
         }
-        for (int m = (ntile >= 2 ? ntile - 2 : 0); m < ntile; ++m) drain(m);
-        {
-            uint32_t v[kCols];
-            tmem_ld16(ocol, v);
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) acc[c] += __uint_as_float(v[c]);
-        }
-        if (valid) {
-            const float scale = (float)green_scale<KIND>();
-            const int64_t base = (row_off + row) * a.nrhs;
-            const int c0 = a.r0 + kCols * half;
-#pragma unroll
-            for (int c = 0; c < kCols; ++c)
-                if (c0 + c < a.nrhs) a.U[base + c0 + c] = scale * acc[c];
-        }
+        flush(ntile);
     }
     if (err) atomicExch(a.status, 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -255,7 +255,6 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
             tx = a.X[row_off + row];
             tl = a.Xlo[row_off + row];
         }
-        const float4 nl = make_float4(-tl.x, -tl.y, -tl.z, 0.f);
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         const int r_first = 32 * (warp & 3), r_last = min(r_first + 31, nrows - 1);
         int s_lo = 0, s_hi = 0;
@@ -294,9 +293,8 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
             if (!mbar_wait(sm_addr(&S.full[s]), (uint32_t)((u / NS) & 1), a.wait_ns)) err = true;
             TcStageC& st = S.st[s];
             const bool adj = (st.tile.flags & TASK_ADJ) != 0;
-            const float cx = st.tile.cen[0], cy = st.tile.cen[1], cz = st.tile.cen[2];
-            const float4 nt = adj ? make_float4(cx - tx.x, cy - tx.y, cz - tx.z, 0.f)
-                                  : make_float4((cx - tx.x) - tl.x, (cy - tx.y) - tl.y, (cz - tx.z) - tl.z, 0.f);
+            float4 nt, nl;
+            tc_frame(tx, tl, st.tile.cen, adj, nt, nl);
             const uint32_t keep = valid ? (st.tile.keep[myslot] >> j0) & kKeepMask : 0u;
             __syncwarp();
             for (int p = lane; p < nsw * kSrcC; p += 32) {

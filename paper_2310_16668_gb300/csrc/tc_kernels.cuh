@@ -302,6 +302,21 @@ template <int KIND, bool ADJ> __device__ __forceinline__ float tc_green(float r2
     return (!ADJ || r2 > 1.17549435e-38f) ? y : 0.f;
 }
 
+// A target's negated coordinates in a chunk's frame (measured from the source
+// box's centre). Touching leaves keep hi and lo apart, and the rounding error
+// of the shift goes to the lo part (as tc_bprep_kernel does for the sources):
+// the difference of two close points is then exact to the lo parts' last bit.
+__device__ __forceinline__ void tc_frame(float4 x, float4 lo, const float* cen, bool adj, float4& nt, float4& nl) {
+    if (adj) {
+        const F2 dx = two_sum(cen[0], -x.x), dy = two_sum(cen[1], -x.y), dz = two_sum(cen[2], -x.z);
+        nt = make_float4(dx.h, dy.h, dz.h, 0.f);
+        nl = make_float4(dx.l - lo.x, dy.l - lo.y, dz.l - lo.z, 0.f);
+    } else {
+        nt = make_float4((cen[0] - x.x) - lo.x, (cen[1] - x.y) - lo.y, (cen[2] - x.z) - lo.z, 0.f);
+        nl = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
 // One source chunk for right-hand sides r0 .. r0+31, laid out as the stage
 // holds it: the B operand in the shared-memory layout of the MMA (element
 // (n, j) at float (j/4)*256 + n*4 + j%4, its lo part 128 floats on; complex:
@@ -367,11 +382,13 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
         const int j = threadIdx.x & 31;
         float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
         if (j < cnt) {
+            const float4 x = X[start + j], o = center[ch];
+            const F2 dx = two_sum(x.x, -o.x), dy = two_sum(x.y, -o.y), dz = two_sum(x.z, -o.z);
             if (threadIdx.x < 32) {
-                const float4 x = X[start + j], o = center[ch];
-                c = make_float4(x.x - o.x, x.y - o.y, x.z - o.z, 0.f);
+                c = make_float4(dx.h, dy.h, dz.h, 0.f);
             } else {
-                c = Xlo[start + j];
+                const float4 l = Xlo[start + j];
+                c = make_float4(l.x + dx.l, l.y + dy.l, l.z + dz.l, 0.f);
             }
         } else if (!CPLX && threadIdx.x < 32) {
             c = make_float4(kFar, kFar, kFar, 0.f);

@@ -169,12 +169,7 @@ __device__ __forceinline__ TcNearTile tc_near_tile(const TcNearRow& r, const Src
     t.kw = r.valid ? st.keep[r.slot] : 0u;
     t.none = REC == kRecNone && __all_sync(0xffffffffu, t.kw == 0u);
     t.some = REC != kRecSym && __any_sync(0xffffffffu, t.kw != 0u && t.kw != all);
-    // the target measured from the source box's centre (the frame of the
-    // chunk's coordinates); touching leaves keep hi and lo apart
-    const float cx = st.cen[0], cy = st.cen[1], cz = st.cen[2];
-    t.nt = adj ? make_float4(cx - r.x.x, cy - r.x.y, cz - r.x.z, 0.f)
-               : make_float4((cx - r.x.x) - r.lo.x, (cy - r.x.y) - r.lo.y, (cz - r.x.z) - r.lo.z, 0.f);
-    t.nl = make_float4(-r.lo.x, -r.lo.y, -r.lo.z, 0.f);
+    tc_frame(r.x, r.lo, st.cen, adj, t.nt, t.nl);
     if (REC != kRecSym && t.kw == 0u) t.nt.x = kFar;
     return t;
 }

@@ -37,7 +37,7 @@ def test_units_match_fp64(kind, n, leaf, dist, nrhs):
     dim = 2 if kind.endswith("2d") else 3
     x = W.points_uniform(n, dim, 71) if dist == "uniform" else clustered(n, dim, 71)
     f = SkelFMM(x, kind, 1e-6, leaf, nrhs_max=nrhs)
-    q = torch.from_numpy(W.charges_normal(n, nrhs, 72)).cuda().float()
+    q = torch.from_numpy(W.charges_normal(x.shape[0], nrhs, 72)).cuda().float()
     u = f.apply(q, "fp32_tc")
     f.device_status()
     ref = f.apply(q.double(), "fp64")

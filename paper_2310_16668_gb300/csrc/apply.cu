@@ -45,6 +45,7 @@
 #include "tc_stored_ring.cuh"
 #include "tc_updown.cuh"
 #include "updown_async.cuh"
+#include "near_sym.cuh"
 
 namespace skel {
 
@@ -108,6 +109,39 @@ T* upload(const std::vector<T>& v, int64_t& bytes) {
     return p;
 }
 
+// Right-hand sides per pass of the symmetric translations: 6.5 and 7.5 FP64
+// operations an interaction (of 3D Laplace) for 1 and 2 columns, against 12 in
+// near_kernel for one and 19 for a pass of up to 8. Two passes of two columns
+// still win, three do not. FP32 stays with near_kernel: there the travelling
+// sums cost as much as an evaluation saves (2D Helmholtz, 8 columns, N = 2^17:
+// 1.22 ms against 1.12).
+constexpr int kSymMaxRhs = 4;
+int sym_columns(int nrhs) { return nrhs == 1 ? 1 : 2; }
+template <class Real>
+bool use_sym(const DevicePlan* dp, int nrhs) {
+    return sizeof(Real) == 8 && dp->n_sym > 0 && nrhs <= kSymMaxRhs;
+}
+
+// the table of log_f64: 1/c, and log c as a multiple of 2^-40 and the rest
+std::vector<double> log_table() {
+    std::vector<double> t(3 * kLogTab);
+    auto value = [](int64_t bits) {
+        double v;
+        std::memcpy(&v, &bits, sizeof(v));
+        return v;
+    };
+    for (int i = 0; i < kLogTab; ++i) {
+        const double lo = value(kLogOff + ((int64_t)i << (52 - kLogBits)));
+        const double hi = value(kLogOff + ((int64_t)(i + 1) << (52 - kLogBits)));
+        const double inv = lo <= 1.0 && 1.0 < hi ? 1.0 : 1.0 / (0.5 * (lo + hi));
+        const long double c = -std::log((long double)inv);
+        t[i] = inv;
+        t[kLogTab + i] = std::ldexp(std::nearbyint(std::ldexp((double)c, 40)), -40);
+        t[2 * kLogTab + i] = (double)(c - (long double)t[kLogTab + i]);
+    }
+    return t;
+}
+
 template <class Real>
 void make_buffers(DevicePlan* dp, const Layout& lay, DeviceBuffers* b) {
     using V = typename RealT<Real>::V4;
@@ -140,7 +174,8 @@ void make_buffers(DevicePlan* dp, const Layout& lay, DeviceBuffers* b) {
     b->Q = dalloc<Real>((size_t)nt * dp->nrhs_max * w, dp->bytes);
     b->U = dalloc<Real>((size_t)nt * dp->nrhs_max * w, dp->bytes);
     const int64_t slots = std::max<int64_t>(dp->n_items, sizeof(Real) == 4 ? dp->tc_n_slots : 0);
-    b->partial = dalloc<Real>((size_t)slots * kChunk * dp->nrhs_max * w, dp->bytes);
+    const int64_t sym = sizeof(Real) == 8 ? dp->sym_slots * 32 * sym_columns(dp->nrhs_max) : 0;
+    b->partial = dalloc<Real>((size_t)std::max(slots * kChunk * dp->nrhs_max, sym) * w, dp->bytes);
 }
 
 void free_buffers(DeviceBuffers* b) {
@@ -357,6 +392,49 @@ NearArgs<Real, CPLX> near_args(DevicePlan* dp, DeviceBuffers* b, const WorkItem*
     return a;
 }
 
+template <int KIND, int RT>
+int sym_pass(const SymArgs<cplx_kind(KIND)>& a, const DevicePlan* dp, cudaStream_t st) {
+    using S = typename Scal<double, cplx_kind(KIND)>::T;
+    sym_kernel<KIND, RT><<<ceil_div(dp->n_sym, kSymWarps), kSymWarps * 32, 0, st>>>(a);
+    CUDA_CHECK(cudaGetLastError());
+    sym_reduce_kernel<S, RT><<<ceil_div(dp->n_chunks * 32, 256), 256, 0, st>>>(
+        dp->sym_ptr, dp->sym_idx, dp->chunk_start, dp->chunk_cnt, dp->n_chunks, a.part, (S*)dp->p64->U, a.nrhs, a.r0);
+    CUDA_CHECK(cudaGetLastError());
+    return 2;
+}
+
+template <int KIND>
+int run_sym_kind(const DevicePlan* dp, int nrhs, cudaStream_t st) {
+    using S = typename Scal<double, cplx_kind(KIND)>::T;
+    const DeviceBuffers* b = dp->p64;
+    SymArgs<cplx_kind(KIND)> a;
+    a.items = dp->sym_items;
+    a.n_items = dp->n_sym;
+    a.chunk_start = dp->chunk_start;
+    a.chunk_cnt = dp->chunk_cnt;
+    a.entry_slot = dp->entry_slot;
+    a.X = (const double4*)b->X;
+    a.Q = (const S*)b->Q;
+    a.part = (S*)b->partial;
+    a.nrhs = nrhs;
+    a.kappa = dp->kappa;
+    a.logtab = dp->logtab;
+    int launches = 0;
+    for (a.r0 = 0; a.r0 < nrhs; a.r0 += sym_columns(nrhs))
+        launches += nrhs == 1 ? sym_pass<KIND, 1>(a, dp, st) : sym_pass<KIND, 2>(a, dp, st);
+    return launches;
+}
+
+// FP64 translations of up to kSymMaxRhs right-hand sides; returns the launches
+int run_sym(const DevicePlan* dp, int nrhs, cudaStream_t st) {
+    switch (dp->kind) {
+        case 0: return run_sym_kind<0>(dp, nrhs, st);
+        case 1: return run_sym_kind<1>(dp, nrhs, st);
+        case 2: return run_sym_kind<2>(dp, nrhs, st);
+        default: return run_sym_kind<3>(dp, nrhs, st);
+    }
+}
+
 // tensor-core translations (real kernels, FP32): the CUDA-core items for
 // the small non-leaf boxes and the reduction of their partial sums (which
 // writes every row of U, zero where no CUDA-core item contributes), then one
@@ -526,6 +604,12 @@ void run_apply(DevicePlan* dp, DeviceBuffers* b, const void* q, void* u, int nrh
         const bool tc = use_tc && (!CPLX || dp->kind == 2) && sizeof(Real) == 4 && dp->n_tc > 0;
         if (tc) {
             launches += run_tc<Real, CPLX>(dp, b, nrhs, st, main_launches);
+            mark(dp, 3, st);
+        } else if (use_sym<Real>(dp, nrhs)) {
+            mark(dp, kMainEvent, st);
+            const int n = run_sym(dp, nrhs, st);
+            main_launches = n / 2;
+            launches += n;
             mark(dp, 3, st);
         } else if (dp->n_items > 0) {
             auto a = near_args<Real, CPLX>(dp, b, dp->items, dp->n_items, nrhs);
@@ -995,6 +1079,24 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
             if (fused > 0) dp->eop2 = upload(eop2, dp->bytes);
         }
         dp->up = upload(up, dp->bytes);
+        // work lists of the row-block kernels, per direction and rows per CTA
+        for (int dir = 0; dir < 2; ++dir)
+            for (int wi = 0; wi < 4; ++wi) {
+                const int rows = 32 << wi;
+                std::vector<int2> w;
+                std::vector<int64_t>& wp = dp->ud_work_ptr[dir][wi];
+                wp.assign(dp->up_level_ptr.size(), 0);
+                for (size_t l = 0; l + 1 < dp->up_level_ptr.size(); ++l) {
+                    wp[l] = (int64_t)w.size();
+                    for (int64_t b = dp->up_level_ptr[l]; b < dp->up_level_ptr[l + 1]; ++b) {
+                        const int nout = dir ? up[b].n - up[b].k : up[b].k;
+                        const int nblk = std::max(dir ? 1 : 0, (nout + rows - 1) / rows);
+                        for (int i = 0; i < nblk; ++i) w.push_back(make_int2((int)b, i * rows));
+                    }
+                }
+                wp.back() = (int64_t)w.size();
+                dp->ud_work[dir][wi] = upload(w, dp->bytes);
+            }
         if (!dp->cplx) {
             // padded FP32 copies of T for the vectorised up/down copies
             std::vector<float> tp, ttp;
@@ -1011,24 +1113,6 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
                 for (int i = 0; i < k; ++i)
                     for (int j = 0; j < r; ++j) ttp[ttpo[b] + j + (size_t)i * ldr] = (float)lay.T[ub.T_off + i + (int64_t)j * k];
             }
-            // work lists of the CTA-wide kernel, per direction and rows per CTA
-            for (int dir = 0; dir < 2; ++dir)
-                for (int wi = 0; wi < 4; ++wi) {
-                    const int rows = 32 << wi;
-                    std::vector<int2> w;
-                    std::vector<int64_t>& wp = dp->ud_work_ptr[dir][wi];
-                    wp.assign(dp->up_level_ptr.size(), 0);
-                    for (size_t l = 0; l + 1 < dp->up_level_ptr.size(); ++l) {
-                        wp[l] = (int64_t)w.size();
-                        for (int64_t b = dp->up_level_ptr[l]; b < dp->up_level_ptr[l + 1]; ++b) {
-                            const int nout = dir ? up[b].n - up[b].k : up[b].k;
-                            const int nblk = std::max(dir ? 1 : 0, (nout + rows - 1) / rows);
-                            for (int i = 0; i < nblk; ++i) w.push_back(make_int2((int)b, i * rows));
-                        }
-                    }
-                    wp.back() = (int64_t)w.size();
-                    dp->ud_work[dir][wi] = upload(w, dp->bytes);
-                }
             dp->ud_tp = upload(tp, dp->bytes);
             dp->ud_ttp = upload(ttp, dp->bytes);
             dp->ud_tp_off = upload(tpo, dp->bytes);
@@ -1075,11 +1159,20 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
                 dp->tc_parts = dalloc<float>((size_t)u.segments * kTcRows * kTcN, dp->bytes);
             }
         }
+        dp->chunk_start = upload(lay.chunk_start, dp->bytes);
+        dp->chunk_cnt = upload(lay.chunk_cnt, dp->bytes);
+        dp->n_chunks = (int64_t)lay.chunk_start.size();
+        dp->n_sym = (int64_t)lay.sym_items.size();
+        dp->sym_slots = lay.sym_slots;
+        if (dp->n_sym > 0) {
+            dp->sym_items = upload(lay.sym_items, dp->bytes);
+            dp->sym_ptr = upload(lay.sym_ptr, dp->bytes);
+            dp->sym_idx = upload(lay.sym_idx, dp->bytes);
+            dp->entry_slot = upload(lay.entry_slot, dp->bytes);
+            if (dp->kind == 0) dp->logtab = upload(log_table(), dp->bytes);
+        }
         if (dp->n_tc > 0 && (!dp->cplx || dp->kind == 2)) {
-            dp->chunk_start = upload(lay.chunk_start, dp->bytes);
-            dp->chunk_cnt = upload(lay.chunk_cnt, dp->bytes);
             dp->chunk_center = upload(lay.chunk_center, dp->bytes);
-            dp->n_chunks = (int64_t)lay.chunk_start.size();
             dp->tc_b = dalloc<float>((size_t)dp->n_chunks * (dp->cplx ? kChunkFloatsC : kChunkFloats), dp->bytes);
         }
         dp->tc_n_slots = lay.tc_n_slots;
@@ -1135,7 +1228,7 @@ void device_plan_destroy(DevicePlan* dp) {
     cudaSetDevice(dp->device);
     void* ptrs[] = {dp->box_off, dp->box_n, dp->box_nslot, dp->slot_start, dp->pos, dp->eop, dp->eop2, dp->up, dp->task_src, dp->task_mask, dp->task_flags, dp->items,
                     dp->part_ptr, dp->part_idx, dp->stage_in, dp->stage_out, dp->mix_items, dp->tc_tiles,
-                    dp->tc_items, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
+                    dp->tc_items, dp->sym_items, dp->sym_ptr, dp->sym_idx, dp->entry_slot, dp->logtab, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
                     dp->tc_part_ptr, dp->tc_part_idx, dp->status,
                     dp->chunk_start, dp->chunk_cnt, dp->chunk_center, dp->tc_b, dp->tc_a, dp->tc_abase,
                     dp->tc_qmask, dp->tc_refs, dp->tc_isym, dp->ud_items_up, dp->ud_items_down,

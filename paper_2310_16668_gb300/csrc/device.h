@@ -56,6 +56,13 @@ struct DevicePlan {
     int64_t tc_n_slots = 0;
     int64_t* tc_part_ptr = nullptr;        // per entry: its partial sums (tensor-core mode)
     int64_t* tc_part_idx = nullptr;
+    // symmetric CUDA-core translations (n_sym = 0: none)
+    SymItem* sym_items = nullptr;
+    int64_t n_sym = 0, sym_slots = 0;
+    int64_t* sym_ptr = nullptr;            // per chunk: its slots
+    int32_t* sym_idx = nullptr;
+    uint8_t* entry_slot = nullptr;
+    double* logtab = nullptr;              // 2D Laplace: table of log_f64
     int64_t* chunk_start = nullptr;        // source chunks (32 entries of one box)
     int32_t* chunk_cnt = nullptr;
     float* chunk_center = nullptr;         // 4 per chunk: its box's centre

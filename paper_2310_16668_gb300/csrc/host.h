@@ -127,6 +127,24 @@ struct WorkItem {                       // one warp: 32 targets x a task range
     int32_t pad;
 };
 
+// One unordered pair (target chunk, source chunks of one box) of the symmetric
+// CUDA-core translations: slot `slot` of 32 rows takes the target chunk's sums,
+// slot + 1 + k those of source chunk schunk + k.
+struct SymItem {                        // 32 bytes
+    uint64_t mask;                      // bit (c*8 + c'): skip target slot c x source slot c'
+    int32_t tchunk, schunk;             // first source chunk
+    int32_t nsrc;                       // source chunks
+    int32_t flags;                      // TASK_ADJ, kSymSelf
+    int32_t slot;
+    int32_t pad;
+};
+static_assert(sizeof(SymItem) == 32, "SymItem layout");
+constexpr int32_t kSymSelf = 2;         // both chunks belong to one box
+// source chunks of an item, at most: one between small boxes, so that a small
+// plan has enough items (a warp needs about 1400 clocks a step by itself), and
+// four between large ones, which halves the slots
+constexpr int sym_chunks(int64_t box_chunks) { return box_chunks <= 8 ? 1 : 4; }
+
 // Tensor-core translations: a CTA owns 128 target rows of one box and streams
 // that box's sources in tiles of 32 (never spanning two tasks).
 constexpr int kTcRows = 128;
@@ -193,6 +211,13 @@ struct Layout {
     std::vector<int64_t> chunk_start;   // first entry of each chunk
     std::vector<int32_t> chunk_cnt;     // entries in it (1..32)
     std::vector<float> chunk_center;    // 4 per chunk: its box's centre (FP32), 0
+    // symmetric CUDA-core translations: items, their slots, and per chunk the
+    // slots that add up to its entries (empty if the tasks are not symmetric)
+    std::vector<SymItem> sym_items;
+    int64_t sym_slots = 0;
+    std::vector<int64_t> sym_ptr;       // chunks + 1
+    std::vector<int32_t> sym_idx;
+    std::vector<uint8_t> entry_slot;    // n_tot: the slot of each entry in its box
     int64_t pairs_direct = 0, pairs_far = 0;
     int64_t pairs_tc = 0;   // kept evaluations inside tensor-core items
 };

@@ -376,6 +376,88 @@ void build_layout(const Plan& p, Layout& lay) {
     // tensor-core items write their rows of U directly
     lay.tc_n_slots = slot;
     to_csr(parts, lay.tc_part_ptr, lay.tc_part_idx);
+
+    // ---- symmetric CUDA-core translations ------------------------------------------
+    // every task has its reverse (the neighbor relations are symmetric and so
+    // are the masks), so each unordered pair of boxes is listed once, from its
+    // lower box, and evaluated for both sides
+    lay.entry_slot.assign(lay.n_tot, 0);
+    for (int64_t b = 0; b < nb; ++b) {
+        if (lay.box_off[b] < 0) continue;
+        const int32_t* ss = &lay.slot_start[b * (kMaxSlots + 1)];
+        for (int j = 0; j < lay.box_nslot[b]; ++j)
+            for (int32_t e = ss[j]; e < ss[j + 1]; ++e) lay.entry_slot[lay.box_off[b] + e] = (uint8_t)j;
+    }
+    lay.sym_items.clear();
+    lay.sym_slots = 0;
+    lay.sym_ptr.assign(lay.chunk_start.size() + 1, 0);
+    lay.sym_idx.clear();
+    auto slots_of = [&](int64_t chunk) {
+        unsigned m = 0;
+        for (int32_t e = 0; e < lay.chunk_cnt[chunk]; ++e) m |= 1u << lay.entry_slot[lay.chunk_start[chunk] + e];
+        return m;
+    };
+    std::vector<uint8_t> chunk_slots(lay.chunk_start.size());
+    for (size_t c = 0; c < chunk_slots.size(); ++c) chunk_slots[c] = (uint8_t)slots_of((int64_t)c);
+    int64_t up_pairs = 0, down_pairs = 0;                   // kept pairs of tasks to higher / lower boxes
+    std::vector<std::pair<int32_t, int32_t>> owner;         // (chunk, slot) in slot order
+    for (int64_t b = 0; b < nb; ++b) {
+        if (lay.box_off[b] < 0) continue;
+        const int64_t tc0 = lay.box_chunk0[b], ntc = (lay.box_n[b] + kTcK - 1) / kTcK;
+        for (int64_t tk = lay.task_ptr[b]; tk < lay.task_ptr[b + 1]; ++tk) {
+            const int64_t src = lay.task_src[tk];
+            const uint64_t mask = lay.task_mask[tk];
+            int64_t kept = 0;
+            for (int i = 0; i < lay.box_nslot[b]; ++i)
+                for (int j = 0; j < lay.box_nslot[src]; ++j)
+                    if (!((mask >> (i * 8 + j)) & 1)) kept += slot_size(b, i) * slot_size(src, j);
+            if (src > b) up_pairs += kept;
+            if (src < b) down_pairs += kept;
+            if (src < b) continue;
+            const int64_t sc0 = lay.box_chunk0[src], nsc = (lay.box_n[src] + kTcK - 1) / kTcK;
+            const int per = sym_chunks(std::max(ntc, nsc));
+            for (int64_t i = 0; i < ntc; ++i) {
+                SymItem it{};
+                it.nsrc = 0;
+                for (int64_t j = src == b ? i : 0; j <= nsc; ++j) {
+                    bool any = false;                        // some pair of slots of the two chunks is kept
+                    if (j < nsc)
+                        for (int c = 0; c < kMaxSlots; ++c)
+                            if (((chunk_slots[tc0 + i] >> c) & 1) &&
+                                (chunk_slots[sc0 + j] & ~(unsigned)(mask >> (8 * c)) & 0xFFu))
+                                any = true;
+                    if (it.nsrc > 0 && (!any || it.nsrc == per)) {
+                        it.slot = (int32_t)lay.sym_slots;
+                        owner.push_back({it.tchunk, it.slot});
+                        for (int k = 0; k < it.nsrc; ++k)
+                            if (it.schunk + k != it.tchunk) owner.push_back({it.schunk + k, it.slot + 1 + k});
+                        lay.sym_slots += 1 + it.nsrc;
+                        if (lay.sym_slots > INT32_MAX - 16) throw Error(-1, "too many translations");
+                        lay.sym_items.push_back(it);
+                        it.nsrc = 0;
+                    }
+                    if (!any) continue;
+                    if (it.nsrc == 0) {
+                        it.mask = mask;
+                        it.tchunk = (int32_t)(tc0 + i);
+                        it.schunk = (int32_t)(sc0 + j);
+                        it.flags = lay.task_flags[tk] | (src == b ? kSymSelf : 0);
+                    }
+                    ++it.nsrc;
+                }
+            }
+        }
+    }
+    if (up_pairs != down_pairs) {
+        lay.sym_items.clear();
+        lay.sym_slots = 0;
+    } else {
+        for (const auto& o : owner) lay.sym_ptr[o.first + 1]++;
+        for (size_t c = 0; c + 1 < lay.sym_ptr.size(); ++c) lay.sym_ptr[c + 1] += lay.sym_ptr[c];
+        lay.sym_idx.resize(owner.size());
+        std::vector<int64_t> at(lay.sym_ptr.begin(), lay.sym_ptr.end() - 1);
+        for (const auto& o : owner) lay.sym_idx[at[o.first]++] = o.second;
+    }
 }
 
 }  // namespace skel
@@ -428,6 +510,7 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
         for (size_t e = 1; e < ptr.size(); ++e) optr.push_back(base + ptr[e]);
         for (int64_t v : idx) oidx.push_back(v + slot_off * kChunk);
     };
+    bool sym = true;                                        // every set has the symmetric items
     for (size_t s = 0; s < ls.size(); ++s) {
         const Layout& l = *ls[s];
         for (int64_t v : l.box_off) m.box_off.push_back(v < 0 ? -1 : v + e0[s]);
@@ -458,6 +541,20 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
             if (it.box >= 0) it.box = (int32_t)(it.box + b0[s]);
             m.tc_items.push_back(it);
         }
+        for (SymItem it : l.sym_items) {
+            it.tchunk = (int32_t)(it.tchunk + c0[s]);
+            it.schunk = (int32_t)(it.schunk + c0[s]);
+            it.slot = (int32_t)(it.slot + m.sym_slots);
+            m.sym_items.push_back(it);
+        }
+        if (m.sym_ptr.empty()) m.sym_ptr.push_back(0);
+        for (size_t c = 1; c < l.sym_ptr.size(); ++c)
+            m.sym_ptr.push_back((int64_t)m.sym_idx.size() + l.sym_ptr[c]);
+        for (int32_t v : l.sym_idx) m.sym_idx.push_back((int32_t)(v + m.sym_slots));
+        m.sym_slots += l.sym_slots;
+        sym &= l.sym_slots > 0;
+        if (m.sym_slots > INT32_MAX) throw Error(-1, "merged plan too large (more than 2^31 partial sums)");
+        m.entry_slot.insert(m.entry_slot.end(), l.entry_slot.begin(), l.entry_slot.end());
         for (int64_t v : l.box_chunk0) m.box_chunk0.push_back(v < 0 ? -1 : v + c0[s]);
         for (int64_t v : l.chunk_start) m.chunk_start.push_back(v + e0[s]);
         m.chunk_cnt.insert(m.chunk_cnt.end(), l.chunk_cnt.begin(), l.chunk_cnt.end());
@@ -465,6 +562,10 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
         m.pairs_direct += l.pairs_direct;
         m.pairs_far += l.pairs_far;
         m.pairs_tc += l.pairs_tc;
+    }
+    if (!sym) {
+        m.sym_items.clear();
+        m.sym_slots = 0;
     }
     if (m.part_ptr.empty()) m.part_ptr.push_back(0);
     if (m.tc_part_ptr.empty()) m.tc_part_ptr.push_back(0);

@@ -46,6 +46,12 @@ template <class S> __device__ __forceinline__ S warp_sum(S v) {
     for (int o = 16; o > 0; o >>= 1) v += shfl_down(v, o);
     return v;
 }
+// the value of another lane
+__device__ __forceinline__ float shfl_from(float v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+__device__ __forceinline__ double shfl_from(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+template <class R> __device__ __forceinline__ Cx<R> shfl_from(Cx<R> v, int lane) {
+    return {shfl_from(v.x, lane), shfl_from(v.y, lane)};
+}
 
 // ---- permutation ------------------------------------------------------------------
 // q (user point order; each right-hand side a column of N) -> Q (entry space,

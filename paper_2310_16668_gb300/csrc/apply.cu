@@ -45,6 +45,7 @@
 #include "tc_stored_ring.cuh"
 #include "tc_updown.cuh"
 #include "updown_async.cuh"
+#include "updown_narrow.cuh"
 #include "near_sym.cuh"
 
 namespace skel {
@@ -289,11 +290,41 @@ int up_down_tc(bool down, DevicePlan* dp, int l, float* X, int nrhs, cudaStream_
     return launches;
 }
 
+template <class S, bool DOWN, int RT>
+void ud_narrow_launch_rt(const DevicePlan* dp, int l, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
+    const std::vector<int64_t>& ptr = dp->ud_work_ptr[DOWN ? 1 : 0][0];
+    const int64_t w0 = ptr[l], n = ptr[l + 1] - w0;
+    if (n <= 0) return;
+    const int2* work = dp->ud_work[DOWN ? 1 : 0][0] + w0;
+    constexpr int th = 32 * kUnWarps;
+    const int ninner = DOWN ? dp->up_level_maxk[l] : dp->up_level_maxr[l];
+    if (ninner <= 2 * un_segment(0))
+        updown_narrow_kernel<S, DOWN, RT, 1><<<ceil_div(n, kUnWarps), th, 0, st>>>(dp->up, work, (int)n, dp->pos, T, X,
+                                                                                  nrhs, conj_op);
+    else
+        updown_narrow_kernel<S, DOWN, RT, kUnWarps><<<(unsigned)n, th, 0, st>>>(dp->up, work, (int)n, dp->pos, T, X,
+                                                                                nrhs, conj_op);
+}
+template <class S, bool DOWN>
+void ud_narrow_launch(const DevicePlan* dp, int l, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
+    if (nrhs == 1) ud_narrow_launch_rt<S, DOWN, 1>(dp, l, nrhs, T, X, conj_op, st);
+    else if (nrhs == 2) ud_narrow_launch_rt<S, DOWN, 2>(dp, l, nrhs, T, X, conj_op, st);
+    else if (nrhs <= 4) ud_narrow_launch_rt<S, DOWN, 4>(dp, l, nrhs, T, X, conj_op, st);
+    else if constexpr (sizeof(S) <= 8) ud_narrow_launch_rt<S, DOWN, 8>(dp, l, nrhs, T, X, conj_op, st);
+}
+
 // one level of the upward or downward pass; warps = 0: the level's setting
 // (autotuned for FP32, else the default rule)
 template <class S>
 void up_down(bool down, const DevicePlan* dp, int l, const S* T, S* X, int nrhs, bool conj_op, cudaStream_t st,
              int warps = 0) {
+    // few right-hand sides: a row per lane instead of a column (every launch
+    // shape below puts 32 columns on the lanes)
+    if (nrhs <= (sizeof(S) <= 8 ? kUnMaxRhs : 4)) {
+        down ? ud_narrow_launch<S, true>(dp, l, nrhs, T, X, conj_op, st)
+             : ud_narrow_launch<S, false>(dp, l, nrhs, T, X, conj_op, st);
+        return;
+    }
     ud_attributes_once<S>();
     const int64_t b0 = dp->up_level_ptr[l], b1 = dp->up_level_ptr[l + 1];
     const int nout = down ? dp->up_level_maxr[l] : dp->up_level_maxk[l];

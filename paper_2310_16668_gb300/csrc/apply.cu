@@ -392,6 +392,7 @@ void permute(bool out, const DevicePlan* dp, const S* src, S* dst, int nrhs, cud
 }
 
 constexpr int64_t kResidentGroups = 4 * 152;   // groups of the on-the-fly kernel that run at a time
+constexpr int32_t kWholeList = INT32_MAX / 2 / kTcGroup * kTcGroup;
 
 constexpr int kProfEvents = 8;   // 7 phase boundaries + the start of the main translation kernel
 constexpr int kMainEvent = 7;
@@ -742,7 +743,7 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
     TcUnit* units = nullptr;                               // one item per unit
     try {
         std::vector<TcUnit> one((size_t)dp->n_tc);
-        for (size_t i = 0; i < one.size(); ++i) one[i] = TcUnit{(int32_t)i, -1, 0, 0, 0, (INT32_MAX / 2 / kTcGroup) * kTcGroup};
+        for (size_t i = 0; i < one.size(); ++i) one[i] = TcUnit{(int32_t)i, -1, 0, 0, 0, kWholeList};
         int64_t unit_bytes = 0;
         units = upload(one, unit_bytes);
         DeviceBuffers* b = dp->p32;
@@ -794,41 +795,50 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
 }
 
 
-// The on-the-fly kernel's units: two items with consecutive rows of one box
-// share a CTA and the tiles it copies; the other items pair up by the length
-// of their lists. Longest first. A plan with few tiles has its long lists cut
-// into parts of whole segments (kTcGroup tiles), so that the chip's 2 x 152
-// resident CTAs get work of about the same length; tc_segments_kernel adds
-// the segments of a cut item. Neither grouping nor cutting changes a result.
+// The on-the-fly kernel's units, longest first. Two items with consecutive
+// rows of one box share a CTA and the tiles it copies, the others pair up by
+// the length of their lists: the CTA's groups then evaluate 32 values a thread
+// between hand-overs. Where the chip's resident CTAs get little work each, and
+// in 2D (short lists), an item per CTA ends sooner: near kernel, pairs against
+// an item per CTA, 3D N = 12,000 (share 12) 176 against 137 us, 20,011 (23) 210
+// against 233, 65,536 (116) 777 against 965 (share: a quarter of the tiles per
+// resident group); 2D N = 65,536 454 against 303 (before tc_log8). There, and for pairs in plans
+// with a little more work, long lists are cut into parts of whole segments
+// (kTcGroup tiles); tc_segments_kernel adds the segments of a cut item.
+// Neither pairing nor cutting changes a result.
+constexpr int64_t kPairShare = 16;             // share from which 3D items share CTAs
+constexpr int64_t kCutShare = 256;             // ... up to which long lists are cut
 struct Units {
     std::vector<TcUnit> units;
     std::vector<int64_t> part0;                            // per item (see TcArgs)
     std::vector<int32_t> split;                            // the cut items
     int64_t segments = 0;                                  // segments of the cut items
 };
-Units make_units(const std::vector<TcItem>& items) {
+Units make_units(const std::vector<TcItem>& items, int dim) {
     auto len = [&](int32_t i) { return items[i].list_hi - items[i].list_lo; };
     int64_t tiles = 0;
     for (size_t i = 0; i < items.size(); ++i) tiles += len((int32_t)i);
-    // a part: about a quarter of what each of the 608 groups gets in all
+    // a part: about a quarter of what each resident group gets in all
     const int64_t share = tiles / (4 * kResidentGroups);
     const int cut = (int)std::max<int64_t>(1, (share + kTcGroup / 2) / kTcGroup) * kTcGroup;
-    const bool small = share < kTcGroup * 4;
-    std::vector<int32_t> order(items.size());
-    for (size_t i = 0; i < items.size(); ++i) order[i] = (int32_t)i;
-    std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return items[x].row_off < items[y].row_off; });
-    std::vector<int32_t> mate(items.size(), -1);
-    for (size_t i = 0; i + 1 < order.size(); ++i) {
-        const TcItem &x = items[order[i]], &y = items[order[i + 1]];
-        if (x.box < 0 || x.box != y.box || x.nrows != kTcRows || y.row_off != x.row_off + kTcRows ||
-            len(order[i]) != len(order[i + 1]))
-            continue;
-        mate[order[i]] = order[i + 1];
-        mate[order[i + 1]] = -2;
-        ++i;
-    }
+    const bool small = share < kCutShare, pairs = dim == 3 && share >= kPairShare;
     Units r;
     r.part0.assign(items.size(), -1);
+    std::vector<int32_t> mate(items.size(), -1);
+    if (pairs) {
+        std::vector<int32_t> order(items.size());
+        for (size_t i = 0; i < items.size(); ++i) order[i] = (int32_t)i;
+        std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return items[x].row_off < items[y].row_off; });
+        for (size_t i = 0; i + 1 < order.size(); ++i) {
+            const TcItem &x = items[order[i]], &y = items[order[i + 1]];
+            if (x.box < 0 || x.box != y.box || x.nrows != kTcRows || y.row_off != x.row_off + kTcRows ||
+                len(order[i]) != len(order[i + 1]))
+                continue;
+            mate[order[i]] = order[i + 1];
+            mate[order[i + 1]] = -2;
+            ++i;
+        }
+    }
     // (item or pair, first tile, tiles) pieces, longest first
     struct Piece {
         int32_t a, b, lo, n;
@@ -851,12 +861,13 @@ Units make_units(const std::vector<TcItem>& items) {
     }
     std::stable_sort(pieces.begin(), pieces.end(),
                      [](const Piece& x, const Piece& y) { return length_class(x.n) > length_class(y.n); });
-    const int whole = (INT32_MAX / 2 / kTcGroup) * kTcGroup;
-    auto count = [&](const Piece& p) { return r.part0[p.a] >= 0 ? cut : whole; };
+    auto count = [&](const Piece& p) { return r.part0[p.a] >= 0 ? cut : kWholeList; };
     const Piece* single = nullptr;
     for (const Piece& p : pieces) {
         if (p.b >= 0) {
             r.units.push_back(TcUnit{p.a, p.b, 1, p.lo, p.lo, count(p)});
+        } else if (!pairs) {
+            r.units.push_back(TcUnit{p.a, -1, 0, p.lo, 0, count(p)});
         } else if (!single || count(*single) != count(p)) {
             if (single) r.units.push_back(TcUnit{single->a, -1, 0, single->lo, 0, count(*single)});
             single = &p;
@@ -1179,7 +1190,7 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
         dp->tc_items = upload(lay.tc_items, dp->bytes);
         dp->n_tc = (int64_t)lay.tc_items.size();
         if (dp->n_tc > 0 && !dp->cplx) {
-            const Units u = make_units(lay.tc_items);
+            const Units u = make_units(lay.tc_items, dp->dim);
             dp->n_units = (int64_t)u.units.size();
             dp->unit0_item = u.units[0].a;
             dp->tc_units = upload(u.units, dp->bytes);

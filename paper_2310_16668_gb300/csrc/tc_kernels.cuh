@@ -7,38 +7,15 @@
 // tile. Before the translations of a 32-column pass, tc_bprep_kernel writes
 // every source chunk (32 consecutive entries of one box) as one contiguous
 // block: its B operand in the MMA's shared-memory layout (K-major, no
-// swizzle, 8 x 16-byte core matrices: 512 bytes between core matrices along
-// K, 128 bytes between groups of 8 right-hand sides), split into TF32 hi and
-// lo, followed by the chunk's coordinates. The CTA is warp-specialised:
-//   * warp 8 (producer; lanes fetch 32 tile descriptors at a time, lane 0
-//     issues): for tile t it waits until data stage t % 6 is free, arms that
-//     stage's "full" mbarrier with the byte count and issues two bulk copies
-//     (cp.async.bulk): the source chunk as the prep kernel laid it out (B hi,
-//     B lo, coordinates; 9 KB) and the tile descriptor, running up to six
-//     tiles ahead of the compute warps;
-//   * warp 9, one thread (MMA issuer): for tile m it waits for "A full" and
-//     issues 12 tcgen05.mma (kind::tf32, M = 128, N = 32, K = 8: hi*hi +
-//     hi*lo + lo*hi for each of 4 K-steps) and commits them to the stage's
-//     "empty" mbarrier;
-//   * warps 0-7 (compute, two threads per target row, 16 sources each): wait
-//     "full", copy their 16 source coordinates once per target slot their
-//     rows fall in (one array per axis, warp-private, so only __syncwarp),
-//     evaluate the kernel block two sources per paired FP32 instruction
-//     (fadd2 / fmul2 / ffma2), split each value into TF32 hi + lo, add the
-//     finished accumulator of tile u - 2 into FP32 registers, write A with
-//     tcgen05.st (TMEM lane = row, column = source) and arrive on "A full".
-// Six data stages and three A buffers keep the bulk copies (issued up to six
-// tiles ahead), the kernel evaluation and the tensor core busy at the same
-// time; the two accumulator tiles alternate, so each tensor-memory
-// accumulation covers one tile only (32 sources) and every longer sum is an
-// FP32 round-to-nearest register sum. The dropped lo*lo term and the
-// truncation of the lo parts are below 2^-21 of each product.
+// swizzle, 8 x 16-byte core matrices), split into TF32 hi and lo, followed by
+// the chunk's coordinates. tc_near.cuh evaluates the kernel and multiplies; this
+// file holds what the tensor-core kernels share and the kernels that read
+// stored values. All of them form the same sum (tc_near.cuh states it) and so
+// give the same bits. The dropped lo*lo term and the truncation of the lo parts
+// are below 2^-21 of each product.
 //
 // Masks: a source that a target row's slot must skip (the regrouped
-// subtractions of Algorithm 2) gets G = 0 in that row: in that slot's copy of
-// the coordinates it sits at 1e30, where r^2 overflows to +inf and the kernel
-// value is exactly 0, so the evaluation itself has no per-source test.
-// Each half of the compute warps drains 16 of the 32 accumulator columns.
+// subtractions of Algorithm 2) gets G = 0 in that row.
 // Waiting threads sleep in the mbarrier (suspend-time hint) rather than spin,
 // and every wait is bounded by wall time (globaltimer, 2 s); on timeout the
 // kernel raises the status word, keeps the protocol going without hanging,
@@ -111,8 +88,8 @@ struct ItemSym {                               // 40 bytes per tensor-core item
 static_assert(sizeof(ItemSym) == 40, "ItemSym layout");
 
 // A unit of the on-the-fly kernel (one CTA): two items, which share their
-// tiles if they hold consecutive rows of one box (equal tile lists), or parts
-// of items' tile lists
+// tiles if they hold consecutive rows of one box (equal tile lists), or one
+// item; a range of their tiles
 struct TcUnit {
     int32_t a, b;                              // items; b = -1: one item
     int32_t shared;

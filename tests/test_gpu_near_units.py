@@ -44,3 +44,22 @@ def test_units_match_fp64(kind, n, leaf, dist, nrhs):
     err = (u.double() - ref).abs().amax(0) / ref.abs().amax(0)
     assert float(err.max()) < 2e-6
     assert torch.equal(f.apply(q, "fp32_tc"), u)
+
+
+def test_log_of_small_distances():
+    """2D, distances of 1e-20 to 1e-17 (r^2 from subnormal to normal FP32, and 0
+    for coincident points). Unit charges, so that a column is single kernel
+    values: r^2 = 1e-40 has a rounding error of 1e-5, 1e-7 of its logarithm, the
+    logarithm rounds to 1e-7 and the 3-pass split to 5e-7."""
+    n = 700
+    x = W.points_uniform(n, 2, 73) * 1e-17
+    x[1::7] = x[::7] + 1e-20
+    x[2::7] = x[::7]
+    f = SkelFMM(x, "laplace2d", 1e-6, n, nrhs_max=33)
+    q = torch.zeros((n, 33), device="cuda")
+    q[torch.arange(33) * 21, torch.arange(33)] = 1.0
+    u = f.apply(q, "fp32_tc")
+    ref = f.apply(q.double(), "fp64")
+    f.device_status()
+    err = (u.double() - ref).abs().amax(0) / ref.abs().amax(0)
+    assert float(err.max()) < 2e-6

@@ -14,29 +14,36 @@ namespace skel {
 // and q = q_r + i q_i is u_r = G_r q_r - G_i q_i, u_i = G_r q_i + G_i q_r, so
 // one real accumulator of 32 columns holds [u_r | u_i] of 16 right-hand sides
 // as G_r B + G_i B' with B = [q_r | q_i] and B' = [-q_i | q_r]
-// (tc_bprep_kernel<true> writes both, TF32 hi + lo). Per tile the MMA issuer
-// adds 12 MMAs of G_r (hi, lo) against B and 12 of G_i against B'. Tensor
-// memory: the accumulators of two tiles (64 columns) and three A buffers of
-// G_r hi, G_r lo, G_i hi, G_i lo (3 x 128 columns): 512 columns, one CTA per
-// SM, so the CTA brings its own latency hiding: 4 compute threads per row
-// (16 compute warps), 8 sources of a tile each.
+// (tc_bprep_kernel<true> writes both, TF32 hi + lo).
+//
+// As in the real kernel (tc_near.cuh) the hi*hi products of a pair of tiles
+// accumulate in D, the small products in L, and hi * [hi | lo] is one MMA into
+// both: 16 MMAs a tile. Pairs alternate between two (D, L); the pair before
+// last is added to the register sums when a pair starts. Tensor memory: two
+// (D, L) (128 columns) and three A buffers of G_r hi, G_r lo, G_i hi, G_i lo
+// (3 x 128): 512 columns, one CTA per SM, so the CTA brings its own latency
+// hiding: 4 compute threads per row (16 compute warps), 8 sources of a tile
+// each. Masks as in tc_near.cuh.
+// Bound by the FP32 pipe: about 60 paired instructions for two values with
+// their split; the MMAs take 16 x 48 of a tile's cycles. FP32, kappa 25, 16
+// right-hand sides, leaves of 128, before (24 MMAs, quadrant selection, a copy
+// of the coordinates per slot) and after: N = 20,011 602 -> 531 us, 4,000
+// 152 -> 138, 1,000 (5 right-hand sides) 60 -> 52; error against complex128
+// 8.4e-7 -> 7.4e-7.
 constexpr int kTcNc = 16;                      // complex right-hand sides per pass
 constexpr uint32_t kTmemColsC = 512;
-constexpr uint32_t kColAc = 64;                // A[b]: G_r hi, G_r lo, G_i hi, G_i lo at 64 + 128 b (+0/32/64/96)
-constexpr int kChunkFloatsC = 4 * 1024 + 2 * 128;
+constexpr uint32_t kColAc = 128;               // A[b]: G_r hi, G_r lo, G_i hi, G_i lo at 128 + 128 b (+0/32/64/96)
+constexpr int kChunkFloatsC = 4 * 1024 + 2 * 96;
 constexpr int kTprC = 4;                       // compute threads per target row
 constexpr int kComputeC = 128 * kTprC;         // compute threads
 constexpr int kSrcC = 32 / kTprC;              // sources of a tile per compute thread
 constexpr int kColsC = kTcN / kTprC;           // accumulator columns per compute thread
 constexpr int kThreadsC = kComputeC + 64;      // + the producer warp and the MMA warp
-constexpr int kSlotFloatsC = 3 * kSrcC;
 struct alignas(128) TcStageC {
-    float bhi[32 * 32];                        // B = [q_r | q_i], TF32 hi
-    float blo[32 * 32];                        //   lo
-    float bphi[32 * 32];                       // B' = [-q_i | q_r], TF32 hi
-    float bplo[32 * 32];                       //   lo
-    float4 xh[32];                             // source coordinates (hi)
-    float4 xl[32];                             // lo parts (touching-leaf tiles)
+    float b[2 * 1024];                         // B = [q_r | q_i], TF32 hi and lo
+    float bp[2 * 1024];                        // B' = [-q_i | q_r], TF32 hi and lo
+    float xh[3 * 32];                          // source coordinates (hi): x, y, z
+    float xl[3 * 32];                          // lo parts (touching-leaf tiles)
     SrcTile tile;                              // the tile's descriptor (its own copy)
 };
 static_assert(offsetof(TcStageC, tile) == kChunkFloatsC * 4, "chunk blob is contiguous in the stage");
@@ -44,7 +51,6 @@ constexpr int kNSC = 6;                        // data stages
 template <int NS>
 struct TcSharedC {
     TcStageC st[NS];
-    float wc[kComputeC / 32][kMaxSlots * kSlotFloatsC];
     float outer[kColsC][kComputeC];
     uint64_t full[NS], afull[NS], empty[NS];
     uint32_t tmem;
@@ -61,64 +67,72 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// sin and cos of two non-negative arguments x below 2^21: x = n pi/2 + y with
-// |y| <= pi/4. n is rounded to nearest by adding 1.5 * 2^23 (the sum's low
-// mantissa bits are then n, so n mod 4 is read from its bits: no conversion
-// instruction); Cody and Waite's reduction with pi/2 as a sum of three floats,
-// the first with 8 significant bits so that n C1 is exact; the Taylor series
-// of sin y to the y^9 term and of cos y to the y^10 term (truncation error
-// below 2e-9 on |y| <= pi/4); then the quadrant n mod 4 maps (sin, cos) to
-// (sin, cos), (cos, -sin), (-sin, -cos), (-cos, sin), the signs as bit flips.
-// FP32 pipe and integer logic only, two arguments per paired instruction.
-__device__ __forceinline__ void tc_sincos2(float2 x, float2& s, float2& c) {
-    constexpr double kHalfPi = 1.57079632679489661923132169163975;
-    constexpr float kC1 = 1.5703125f;
-    constexpr float kC2 = (float)(kHalfPi - 1.5703125);
-    constexpr float kC3 = (float)(kHalfPi - 1.5703125 - (double)kC2);
-    constexpr float kTwoOverPi = (float)(1.0 / kHalfPi);
+// (-1)^n sin x and (-1)^n cos x of two non-negative arguments x up to 2^21,
+// with n = x / pi rounded to nearest, whose parity comes back in bit 0 of nx
+// and ny: x = n pi + y with |y| <= pi/2. n is rounded by adding 1.5 * 2^23 (the
+// sum's low mantissa bits are then n: no conversion instruction); Cody and
+// Waite's reduction with pi as a sum of three floats, the first with 9
+// significant bits so that n C1 is exact; the Taylor series of sin y to the
+// y^13 term (truncation below 7e-10 on |y| <= pi/2) and of cos y to the y^14
+// term (below 7e-11). Reducing by pi instead of pi/2 takes three more
+// coefficients but no choice between the two series and one sign for both,
+// which the caller puts on the common factor 1/r: two integer instructions a
+// value instead of ten. FP32 pipe only, two arguments per paired instruction.
+__device__ __forceinline__ void tc_sincos2(float2 x, float2& s, float2& c, uint32_t& nx, uint32_t& ny) {
+    constexpr double kPi = 3.14159265358979323846264338327950;
+    constexpr float kC1 = 3.140625f;
+    constexpr float kC2 = (float)(kPi - 3.140625);
+    constexpr float kC3 = (float)(kPi - 3.140625 - (double)kC2);
     constexpr float kRound = 12582912.0f;      // 1.5 * 2^23
-    const float2 t = __ffma2_rn(x, tc_f2(kTwoOverPi), tc_f2(kRound));
+    const float2 t = __ffma2_rn(x, tc_f2((float)(1.0 / kPi)), tc_f2(kRound));
     const float2 mn = __ffma2_rn(t, tc_f2(-1.f), tc_f2(kRound));   // -n (exact)
     float2 y = __ffma2_rn(mn, tc_f2(kC1), x);
     y = __ffma2_rn(mn, tc_f2(kC2), y);
     y = __ffma2_rn(mn, tc_f2(kC3), y);
     const float2 z = __fmul2_rn(y, y);
-    float2 ps = __ffma2_rn(z, tc_f2((float)(1.0 / 362880.0)), tc_f2((float)(-1.0 / 5040.0)));
+    float2 ps = __ffma2_rn(z, tc_f2((float)(1.0 / 6227020800.0)), tc_f2((float)(-1.0 / 39916800.0)));
+    ps = __ffma2_rn(z, ps, tc_f2((float)(1.0 / 362880.0)));
+    ps = __ffma2_rn(z, ps, tc_f2((float)(-1.0 / 5040.0)));
     ps = __ffma2_rn(z, ps, tc_f2((float)(1.0 / 120.0)));
     ps = __ffma2_rn(z, ps, tc_f2((float)(-1.0 / 6.0)));
-    const float2 sy = __ffma2_rn(__fmul2_rn(y, z), ps, y);
-    float2 pc = __ffma2_rn(z, tc_f2((float)(-1.0 / 3628800.0)), tc_f2((float)(1.0 / 40320.0)));
+    s = __ffma2_rn(__fmul2_rn(y, z), ps, y);
+    float2 pc = __ffma2_rn(z, tc_f2((float)(-1.0 / 87178291200.0)), tc_f2((float)(1.0 / 479001600.0)));
+    pc = __ffma2_rn(z, pc, tc_f2((float)(-1.0 / 3628800.0)));
+    pc = __ffma2_rn(z, pc, tc_f2((float)(1.0 / 40320.0)));
     pc = __ffma2_rn(z, pc, tc_f2((float)(-1.0 / 720.0)));
     pc = __ffma2_rn(z, pc, tc_f2((float)(1.0 / 24.0)));
     pc = __ffma2_rn(z, pc, tc_f2(-0.5f));
-    const float2 cy = __ffma2_rn(z, pc, tc_f2(1.0f));
-    const uint32_t qx = __float_as_uint(t.x), qy = __float_as_uint(t.y);
-    // sign of sin: bit 1 of n; sign of cos: bit 1 of n + 1
-    const uint32_t ssx = (qx << 30) & 0x80000000u, ssy = (qy << 30) & 0x80000000u;
-    const uint32_t csx = ((qx + 1u) << 30) & 0x80000000u, csy = ((qy + 1u) << 30) & 0x80000000u;
-    s.x = __uint_as_float(__float_as_uint((qx & 1u) ? cy.x : sy.x) ^ ssx);
-    c.x = __uint_as_float(__float_as_uint((qx & 1u) ? sy.x : cy.x) ^ csx);
-    s.y = __uint_as_float(__float_as_uint((qy & 1u) ? cy.y : sy.y) ^ ssy);
-    c.y = __uint_as_float(__float_as_uint((qy & 1u) ? sy.y : cy.y) ^ csy);
+    c = __ffma2_rn(z, pc, tc_f2(1.0f));
+    nx = __float_as_uint(t.x);
+    ny = __float_as_uint(t.y);
+    asm volatile("" : "+r"(nx), "+r"(ny));     // (as in tc_log8)
 }
 
-// e^{i kappa r} / r without its 1/(4 pi), for CNT sources (as tc_eval16):
-// the reciprocal square root as in the real path (0 for masked sources and,
-// on touching leaves, for r^2 <= FLT_MIN), r = r^2 / r corrected by one
-// Newton step, then tc_sincos2 of kappa r. A zero reciprocal gives
-// kappa r = 0 (not the NaN of +inf * 0), so masked sources have the value 0.
-template <bool ADJ, int CNT, int AX>
-__device__ __forceinline__ void tc_ceval(const float* c, const float4* xl, int j0, float4 nt, float4 nl,
-                                         float kappa, uint32_t* grh, uint32_t* grl, uint32_t* gih, uint32_t* gil) {
+// e^{i kappa r} / r without its 1/(4 pi) for 8 sources (coordinates at x: 32
+// floats per axis, lo parts 96 floats on), split into TF32 hi and lo: the
+// reciprocal square root as in the real path (0 at kFar and, on touching
+// leaves, for r^2 <= FLT_MIN), r = r^2 / r corrected by one Newton step, then
+// tc_sincos2 of kappa r. A zero reciprocal makes r a NaN or 0; the minimum
+// with 2^21 turns that (and only that: kappa r stays far below) into a finite
+// argument, whose sine and cosine the zero reciprocal then cancels.
+// kb: the row's kept sources (bit per source), used if CUT.
+template <bool ADJ, bool CUT>
+__device__ __forceinline__ void tc_ceval(const float* x, float4 nt, float4 nl, float kappa, uint32_t kb, uint32_t* grh,
+                                         uint32_t* grl, uint32_t* gih, uint32_t* gil) {
+    constexpr int AX = 32, LO = 96;
     const float2 ntx = tc_f2(nt.x), nty = tc_f2(nt.y), ntz = tc_f2(nt.z);
-    float2 nlx, nly, nlz;
-    if (ADJ) nlx = tc_f2(nl.x), nly = tc_f2(nl.y), nlz = tc_f2(nl.z);
-    const float2 m1 = tc_f2(-1.f), split = tc_f2(8193.f), kap = tc_f2(kappa), half = tc_f2(0.5f);
+    const float2 m1 = tc_f2(-1.f), split = tc_f2(8193.f), kap = tc_f2(kappa);
 #pragma unroll
-    for (int q = 0; q < CNT / 4; ++q) {
-        const float4 X = *reinterpret_cast<const float4*>(&c[4 * q]);
-        const float4 Y = *reinterpret_cast<const float4*>(&c[AX + 4 * q]);
-        const float4 Z = *reinterpret_cast<const float4*>(&c[2 * AX + 4 * q]);
+    for (int q = 0; q < kSrcC / 4; ++q) {
+        const float4 X = *reinterpret_cast<const float4*>(x + 4 * q);
+        const float4 Y = *reinterpret_cast<const float4*>(x + AX + 4 * q);
+        const float4 Z = *reinterpret_cast<const float4*>(x + 2 * AX + 4 * q);
+        float4 LX, LY, LZ;
+        if (ADJ) {
+            LX = *reinterpret_cast<const float4*>(x + LO + 4 * q);
+            LY = *reinterpret_cast<const float4*>(x + LO + AX + 4 * q);
+            LZ = *reinterpret_cast<const float4*>(x + LO + 2 * AX + 4 * q);
+        }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int jj = 4 * q + 2 * h;
@@ -126,24 +140,30 @@ __device__ __forceinline__ void tc_ceval(const float* c, const float4* xl, int j
             float2 dy = __fadd2_rn(h ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y), nty);
             float2 dz = __fadd2_rn(h ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y), ntz);
             if (ADJ) {
-                const float4 l0 = xl[j0 + jj], l1 = xl[j0 + jj + 1];
-                dx = __fadd2_rn(dx, __fadd2_rn(make_float2(l0.x, l1.x), nlx));
-                dy = __fadd2_rn(dy, __fadd2_rn(make_float2(l0.y, l1.y), nly));
-                dz = __fadd2_rn(dz, __fadd2_rn(make_float2(l0.z, l1.z), nlz));
+                dx = __fadd2_rn(dx, __fadd2_rn(h ? make_float2(LX.z, LX.w) : make_float2(LX.x, LX.y), tc_f2(nl.x)));
+                dy = __fadd2_rn(dy, __fadd2_rn(h ? make_float2(LY.z, LY.w) : make_float2(LY.x, LY.y), tc_f2(nl.y)));
+                dz = __fadd2_rn(dz, __fadd2_rn(h ? make_float2(LZ.z, LZ.w) : make_float2(LZ.x, LZ.y), tc_f2(nl.z)));
             }
             float2 r2 = __fmul2_rn(dx, dx);
             r2 = __ffma2_rn(dy, dy, r2);
             r2 = __ffma2_rn(dz, dz, r2);
-            const float2 ri = make_float2(tc_green<1, ADJ>(r2.x), tc_green<1, ADJ>(r2.y));
+            float2 ri = make_float2(tc_green<1, ADJ>(r2.x), tc_green<1, ADJ>(r2.y));
             float2 r = __fmul2_rn(r2, ri);
-            r = __ffma2_rn(__fmul2_rn(half, ri), __ffma2_rn(__fmul2_rn(r, m1), r, r2), r);
+            r = __ffma2_rn(r, __ffma2_rn(r, __fmul2_rn(ri, tc_f2(-0.5f)), tc_f2(0.5f)), r);
             float2 kr = __fmul2_rn(kap, r);
-            kr.x = ri.x > 0.f ? kr.x : 0.f;
-            kr.y = ri.y > 0.f ? kr.y : 0.f;
+            kr.x = fminf(kr.x, 2097152.f);
+            kr.y = fminf(kr.y, 2097152.f);
+            if (CUT) {
+                ri.x = (kb >> jj) & 1u ? ri.x : 0.f;
+                ri.y = (kb >> (jj + 1)) & 1u ? ri.y : 0.f;
+            }
             float2 sn, cs;
-            tc_sincos2(kr, sn, cs);
+            uint32_t nx, ny;
+            tc_sincos2(kr, sn, cs, nx, ny);
+            ri.x = __uint_as_float(__float_as_uint(ri.x) ^ (nx << 31));
+            ri.y = __uint_as_float(__float_as_uint(ri.y) ^ (ny << 31));
             const float2 gR = __fmul2_rn(cs, ri), gI = __fmul2_rn(sn, ri);
-            // Veltkamp's split of both parts (as tc_eval16)
+            // Veltkamp's split of both parts (as tc_split_store)
             const float2 tR = __fmul2_rn(gR, split), tI = __fmul2_rn(gI, split);
             const float2 hR = __ffma2_rn(__ffma2_rn(gR, m1, tR), m1, tR);
             const float2 hI = __ffma2_rn(__ffma2_rn(gI, m1, tI), m1, tI);
@@ -203,7 +223,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
                 if (lane == 0) {
                     const uint32_t bar = sm_addr(&S.full[s]);
                     mbar_arrive_tx(bar, 4u * kChunkFloatsC + 64u);
-                    bulk_g2s_hint(sm_addr(S.st[s].bhi), a.B + (int64_t)chunk * kChunkFloatsC, 4u * kChunkFloatsC, bar,
+                    bulk_g2s_hint(sm_addr(S.st[s].b), a.B + (int64_t)chunk * kChunkFloatsC, 4u * kChunkFloatsC, bar,
                                   l2_evict_last());
                     bulk_g2s_hint(sm_addr(&S.st[s].tile), a.tiles + list_lo + t, 64u, bar, l2_evict_first());
                     if (hold && !mbar_wait(bar, 0u, a.wait_ns)) err = true;
@@ -218,26 +238,24 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
     } else if (warp == kComputeC / 32 + 1) {
         // ---------------- MMA issuer (one thread) ----------------
         if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
-                                   ((128u >> 4) << 24);
+            const uint32_t idesc32 =
+                (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(kTcN >> 3) << 17) | ((128u >> 4) << 24);
+            const uint32_t idesc64 =
+                (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(2 * kTcN >> 3) << 17) | ((128u >> 4) << 24);
             for (int m = 0; m < ntile; ++m) {
                 const int s = m % NS, ab = m % kNA;
                 if (!mbar_wait(sm_addr(&S.afull[s]), (uint32_t)((m / NS) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t bh = sm_addr(S.st[s].bhi), bl = sm_addr(S.st[s].blo);
-                const uint32_t bph = sm_addr(S.st[s].bphi), bpl = sm_addr(S.st[s].bplo);
-                const uint32_t d = tbase + kColD + 32u * (m & 1);
+                const uint32_t b0 = smem_desc_lo(sm_addr(S.st[s].b)), bp0 = smem_desc_lo(sm_addr(S.st[s].bp));
+                const uint32_t d = tbase + 64u * ((uint32_t)(m >> 1) & 1u), l = d + 32u;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const uint32_t arh = tbase + kColAc + 128u * ab + 8u * k, arl = arh + 32u;
-                    const uint32_t aih = arh + 64u, ail = arh + 96u;
-                    const uint32_t ko = 2u * kBLbo * k;
-                    mma_tf32(d, arh, smem_desc(bh + ko), idesc, k > 0 ? 1u : 0u);
-                    mma_tf32(d, arh, smem_desc(bl + ko), idesc, 1u);
-                    mma_tf32(d, arl, smem_desc(bh + ko), idesc, 1u);
-                    mma_tf32(d, aih, smem_desc(bph + ko), idesc, 1u);
-                    mma_tf32(d, aih, smem_desc(bpl + ko), idesc, 1u);
-                    mma_tf32(d, ail, smem_desc(bph + ko), idesc, 1u);
+                    const uint32_t ar = tbase + kColAc + 128u * ab + 8u * k, ai = ar + 64u;
+                    const uint32_t db = b0 + kDescStep * k, dbp = bp0 + kDescStep * k;
+                    mma_tf32_lo(d, ar, db, idesc64, true);             // D, L += G_r hi [hi | lo]
+                    mma_tf32_lo(l, ar + 32u, db, idesc32, true);       // L += G_r lo hi
+                    mma_tf32_lo(d, ai, dbp, idesc64, true);
+                    mma_tf32_lo(l, ai + 32u, dbp, idesc32, true);
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.empty[s])) : "memory");
@@ -256,70 +274,88 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
             tl = a.Xlo[row_off + row];
         }
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-        const int r_first = 32 * (warp & 3), r_last = min(r_first + 31, nrows - 1);
-        int s_lo = 0, s_hi = 0;
-        for (int c = 1; c < nslot; ++c) {
-            if (r_first >= itp->slot_start[c]) s_lo = c;
-            if (r_last >= itp->slot_start[c]) s_hi = c;
-        }
-        const int nsw = max(1, s_hi - s_lo + 1);
-        const int myloc = min(max(myslot - s_lo, 0), kMaxSlots - 1);
-        float* wc = S.wc[warp];
-        constexpr uint32_t kKeepMask = (1u << kSrcC) - 1u;
         const int j0 = kSrcC * quarter;
+        const uint32_t dcol = tbase + lane_off + (uint32_t)(kColsC * quarter);
         float acc[kColsC];
 #pragma unroll
         for (int c = 0; c < kColsC; ++c) {
             acc[c] = 0.f;
             S.outer[c][tid] = 0.f;
         }
-        auto drain = [&](int m) {
-            if (!mbar_wait(sm_addr(&S.empty[m % NS]), (uint32_t)((m / NS) & 1), a.wait_ns)) err = true;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        auto clear = [&]() {                                   // this thread's columns of both (D, L)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tmem_st8(dcol + 32u * i, zero);
+        };
+        auto add = [&](uint32_t taddr) {
             uint32_t v[kColsC];
-            tmem_ld8(tbase + lane_off + kColD + 32u * (m & 1) + (uint32_t)(kColsC * quarter), v);
+            tmem_ld8(taddr, v);
 #pragma unroll
             for (int c = 0; c < kColsC; ++c) acc[c] += __uint_as_float(v[c]);
-            if (m % kTcOuter == kTcOuter - 1) {
+        };
+        // tile m's MMAs are done: asked for early, settled when it matters
+        auto ask = [&](int m) { return mbar_test(sm_addr(&S.empty[m % NS]), (uint32_t)((m / NS) & 1)); };
+        auto settle = [&](uint32_t early, int m) {
+            if (!mbar_settle(early, sm_addr(&S.empty[m % NS]), (uint32_t)((m / NS) & 1), a.wait_ns)) err = true;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        };
+        // everything accumulated in tensor memory before tile u of the group
+        // that starts at s0, to the outer sums
+        auto flush = [&](int u, int s0) {
+            if (u <= s0) return;
+            settle(ask(u - 1), u - 1);
+            const int np = (u - s0 + 1) / 2;
+            for (int p = max(np - 2, 0); p < np; ++p) add(dcol + 64u * ((uint32_t)p & 1u));
+            add(dcol + 32u);
+            add(dcol + 96u);
 #pragma unroll
-                for (int c = 0; c < kColsC; ++c) {
-                    S.outer[c][tid] += acc[c];
-                    acc[c] = 0.f;
-                }
+            for (int c = 0; c < kColsC; ++c) {
+                S.outer[c][tid] += acc[c];
+                acc[c] = 0.f;
             }
         };
+        clear();
+        uint32_t landed = 0u;                                  // the next tile's copies, asked for early
         for (int u = 0; u < ntile; ++u) {
             const int s = u % NS;
-            if (!mbar_wait(sm_addr(&S.full[s]), (uint32_t)((u / NS) & 1), a.wait_ns)) err = true;
-            TcStageC& st = S.st[s];
+            if (!mbar_settle(landed, sm_addr(&S.full[s]), (uint32_t)((u / NS) & 1), a.wait_ns)) err = true;
+            landed = mbar_test(sm_addr(&S.full[(u + 1) % NS]), (uint32_t)(((u + 1) / NS) & 1));
+            const uint32_t early = u >= 3 ? ask(u - 3) : 0u;
+            const TcStageC& st = S.st[s];
             const bool adj = (st.tile.flags & TASK_ADJ) != 0;
+            const uint32_t all = st.tile.cnt >= 32 ? 0xFFFFFFFFu : (1u << (st.tile.cnt & 31)) - 1u;
             float4 nt, nl;
             tc_frame(tx, tl, st.tile.cen, adj, nt, nl);
-            const uint32_t keep = valid ? (st.tile.keep[myslot] >> j0) & kKeepMask : 0u;
-            __syncwarp();
-            for (int p = lane; p < nsw * kSrcC; p += 32) {
-                const int ls = p / kSrcC, jj = p % kSrcC;
-                const float4 v = st.xh[j0 + jj];
-                const bool kept = ((st.tile.keep[s_lo + ls] >> (j0 + jj)) & 1u) != 0u;
-                float* d = wc + ls * kSlotFloatsC + jj;
-                d[0] = kept ? v.x : kFar;
-                d[kSrcC] = kept ? v.y : kFar;
-                d[2 * kSrcC] = kept ? v.z : kFar;
-            }
-            __syncwarp();
-            if (u >= 2) drain(u - 2);
-            const uint32_t acol = tbase + lane_off + kColAc + 128u * (u % kNA) + (uint32_t)j0;
-            const float* c = wc + myloc * kSlotFloatsC;
-            const bool none = __all_sync(0xffffffffu, keep == 0);
+            const uint32_t kb = valid ? (st.tile.keep[myslot] >> j0) & 0xFFu : 0u;
+            const bool none = __all_sync(0xffffffffu, kb == 0u);
+            const bool cut = __any_sync(0xffffffffu, kb != 0u && kb != (all >> j0 & 0xFFu));
+            if (kb == 0u) nt.x = kFar;                         // the row keeps none of these sources
             uint32_t grh[kSrcC], grl[kSrcC], gih[kSrcC], gil[kSrcC];
             if (none) {
 #pragma unroll
                 for (int jj = 0; jj < kSrcC; ++jj) grh[jj] = grl[jj] = gih[jj] = gil[jj] = 0u;
             } else if (adj) {
-                tc_ceval<true, kSrcC, kSrcC>(c, st.xl, j0, nt, nl, a.kappa, grh, grl, gih, gil);
+                if (cut) tc_ceval<true, true>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
+                else tc_ceval<true, false>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
             } else {
-                tc_ceval<false, kSrcC, kSrcC>(c, st.xl, j0, nt, nl, a.kappa, grh, grl, gih, gil);
+                if (cut) tc_ceval<false, true>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
+                else tc_ceval<false, false>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
             }
+            const int g = u & (kTcOuter - 1);                  // tile of the group
+            if (u > 0 && g == 0) {
+                flush(u, u - kTcOuter);
+                clear();
+            } else if (u >= 3) {
+                // A buffer u % 3 was last read by MMA(u - 3)
+                settle(early, u - 3);
+                // the pair two before the one that starts here, which restarts its D
+                if (g >= 4 && !(g & 1)) {
+                    const uint32_t dc = dcol + 64u * ((uint32_t)(g >> 1) & 1u);
+                    add(dc);
+                    tmem_st8(dc, zero);
+                }
+            }
+            const uint32_t acol = tbase + lane_off + kColAc + 128u * (u % kNA) + (uint32_t)j0;
             tmem_st8(acol, grh);
             tmem_st8(acol + 32u, grl);
             tmem_st8(acol + 64u, gih);
@@ -328,9 +364,9 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(sm_addr(&S.afull[s]));
         }
-        for (int m = (ntile >= 2 ? ntile - 2 : 0); m < ntile; ++m) drain(m);
+        flush(ntile, ntile > 0 ? (ntile - 1) & ~(kTcOuter - 1) : 0);
 #pragma unroll
-        for (int c = 0; c < kColsC; ++c) acc[c] += S.outer[c][tid];
+        for (int c = 0; c < kColsC; ++c) acc[c] = S.outer[c][tid];
         if (valid) {
             // quarter q holds columns 8q .. 8q + 7: real parts of right-hand
             // sides r0 + 8 (q & 1) .. + 7 (q < 2), their imaginary parts (q >= 2)

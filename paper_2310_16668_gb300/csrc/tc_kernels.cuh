@@ -161,6 +161,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     }
 }
 
+// An early look at a barrier whose phase is needed later: a wait takes 150 to
+// 300 clocks of a busy SM even when the phase is complete, so it is asked for
+// before work that does not need it and settled after that work.
+__device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                 " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok) : "r"(bar), "r"(parity));
+    return ok;
+}
+__device__ __forceinline__ bool mbar_settle(uint32_t early, uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+    bool ok = true;
+    if (!__all_sync(0xffffffffu, early != 0u)) ok = mbar_wait(bar, parity, limit_ns);
+    asm volatile("" ::: "memory");
+    return ok;
+}
+
 // Test hook of the bounded waits (TcArgs::withhold_item): before the first
 // tile's copies the producer waits until the compute warps have given up
 // waiting for them and arrived on "A full"; then it issues the copies and
@@ -205,12 +221,11 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst, const void* src, uin
 
 // B operand layout (K-major, no swizzle): core matrix = 8 columns x 4 sources
 // (16 bytes per row); the groups of 8 columns of one 4-source slab are
-// contiguous (SBO = 128 B) and slabs follow along K (LBO). Real kernels: 64
-// columns per slab, the 32 right-hand sides' TF32 hi parts, then their lo
-// parts (LBO = 1 KB; the lo parts alone start 512 B on). Complex kernels: 32
-// columns per slab, hi and lo parts as separate 4 KB operands (LBO = 512 B).
+// contiguous (SBO = 128 B) and slabs follow along K (LBO). A chunk's slab has
+// 64 columns: 32 TF32 hi parts, then their lo parts (LBO = 1 KB; the lo parts
+// alone start 512 B on). The skeleton GEMMs' slabs have 32 (LBO = 512 B).
 constexpr uint32_t kBLbo = 512, kBSbo = 128;
-constexpr uint32_t kBLboReal = 1024, kBLoPart = 512;
+constexpr uint32_t kBLboChunk = 1024, kBLoPart = 512;
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
@@ -220,13 +235,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     return d;                                        // base offset 0, no swizzle
 }
 
-// the low word of the descriptor of a real chunk's B operand at addr; per
+// the low word of the descriptor of a chunk's B operand at addr; per
 // K-step of 8 sources add kDescStep, for the lo columns add kDescLoPart
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) {
-    return ((addr >> 4) & 0x3FFF) | (((kBLboReal >> 4) & 0x3FFF) << 16);
+    return ((addr >> 4) & 0x3FFF) | (((kBLboChunk >> 4) & 0x3FFF) << 16);
 }
 constexpr uint32_t kDescHi = ((kBSbo >> 4) & 0x3FFF) | (1u << 14);   // SBO; descriptor version
-constexpr uint32_t kDescStep = 2u * kBLboReal / 16u, kDescLoPart = kBLoPart / 16u;
+constexpr uint32_t kDescStep = 2u * kBLboChunk / 16u, kDescLoPart = kBLoPart / 16u;
 
 // d (+)= A B^T; acc: accumulate (else overwrite d)
 __device__ __forceinline__ void mma_tf32_lo(uint32_t d, uint32_t a, uint32_t desc_lo, uint32_t idesc, bool acc) {
@@ -296,9 +311,8 @@ __device__ __forceinline__ void tc_frame(float4 x, float4 lo, const float* cen, 
 
 // One source chunk for right-hand sides r0 .. r0+31, laid out as the stage
 // holds it: the B operand in the shared-memory layout of the MMA (element
-// (n, j) at float (j/4)*256 + n*4 + j%4, its lo part 128 floats on; complex:
-// (j/4)*128, the lo parts 1024 floats on), split into TF32 hi (rounded to
-// nearest) and lo = q - hi, then the chunk's 32 source coordinates (hi part
+// (n, j) at float (j/4)*256 + n*4 + j%4, its lo part 128 floats on), split
+// into TF32 hi (rounded to nearest) and lo = q - hi, then the chunk's 32 source coordinates (hi part
 // minus the box centre: FP32 then resolves them to the box size, not to the
 // domain size) and their lo parts; entries past the chunk and columns past
 // nrhs are zero.
@@ -313,7 +327,7 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
                                                        const float* __restrict__ Q, int nrhs, int r0,
                                                        const float4* __restrict__ X, const float4* __restrict__ Xlo,
                                                        const float4* __restrict__ center, float* __restrict__ B) {
-    constexpr int kBlob = CPLX ? 4 * 1024 + 2 * 128 : kChunkFloats;
+    constexpr int kBlob = CPLX ? 4 * 1024 + 2 * 96 : kChunkFloats;
     constexpr int kXoff = CPLX ? 4096 : 2048;
     const int64_t ch = blockIdx.x;
     const int n = threadIdx.x & 31, jq = threadIdx.x >> 5;
@@ -345,13 +359,8 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
         h.z = __uint_as_float(to_tf32(x[2]));
         h.w = __uint_as_float(to_tf32(x[3]));
         l = make_float4(x[0] - h.x, x[1] - h.y, x[2] - h.z, x[3] - h.w);
-        if constexpr (CPLX) {
-            *reinterpret_cast<float4*>(blob + 2048 * part + jq * 128 + n * 4) = h;
-            *reinterpret_cast<float4*>(blob + 2048 * part + 1024 + jq * 128 + n * 4) = l;
-        } else {
-            *reinterpret_cast<float4*>(blob + jq * 256 + n * 4) = h;
-            *reinterpret_cast<float4*>(blob + jq * 256 + 128 + n * 4) = l;
-        }
+        *reinterpret_cast<float4*>(blob + 2048 * part + jq * 256 + n * 4) = h;
+        *reinterpret_cast<float4*>(blob + 2048 * part + jq * 256 + 128 + n * 4) = l;
     }
     // the chunk's coordinates: hi parts measured from the box centre, then
     // the lo parts (zero past cnt)
@@ -367,17 +376,13 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
                 const float4 l = Xlo[start + j];
                 c = make_float4(l.x + dx.l, l.y + dy.l, l.z + dz.l, 0.f);
             }
-        } else if (!CPLX && threadIdx.x < 32) {
+        } else if (threadIdx.x < 32) {
             c = make_float4(kFar, kFar, kFar, 0.f);
         }
-        if constexpr (CPLX) {
-            reinterpret_cast<float4*>(blob + kXoff)[threadIdx.x] = c;
-        } else {
-            float* d = blob + kXoff + (threadIdx.x >> 5) * 96 + j;
-            d[0] = c.x;
-            d[32] = c.y;
-            d[64] = c.z;
-        }
+        float* d = blob + kXoff + (threadIdx.x >> 5) * 96 + j;
+        d[0] = c.x;
+        d[32] = c.y;
+        d[64] = c.z;
     }
 }
 

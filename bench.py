@@ -41,10 +41,10 @@ SM_COUNT = 152
 MUFU_PER_SM_CLK = 16      # MUFU (rsqrt) results per SM per clock
 FP32_PER_SM_CLK = 128     # FP32 lane operations per SM per clock (a paired instruction counts as two)
 # FP32 operations per complex kernel evaluation in tc_cnear_kernel, counted
-# from its source (tc_ceval16 + tc_sincos2): differences 3, r^2 3, r with one
-# Newton step 5, kappa r 1, reduction 3 + 2, z 1, sin 5, cos 5, G_r / G_i 2,
+# from its source (tc_ceval + tc_sincos2): differences 3, r^2 3, r with one
+# Newton step 5, kappa r 1, reduction 5, z 1, sin 7, cos 7, G_r / G_i 2,
 # TF32 split 8 (touching-leaf tiles add 9, not counted)
-FP32_OPS_HELMHOLTZ_TC = 38
+FP32_OPS_HELMHOLTZ_TC = 42
 
 
 # --workload name -> workload in paper_2310_16668_gb300.workloads
@@ -153,7 +153,7 @@ def kernel_source_sha(kernel: str = "") -> str:
     the structures they read; the complex tensor-core kernel adds its own
     header); a committed traffic figure counts only while it matches."""
     h = hashlib.sha256()
-    files = ("skel_kernels.cuh", "tc_kernels.cuh", "host.h")
+    files = ("skel_kernels.cuh", "tc_kernels.cuh", "tc_near.cuh", "host.h")
     if kernel == "tc_cnear_kernel":
         files += ("tc_complex.cuh",)
     for f in files:

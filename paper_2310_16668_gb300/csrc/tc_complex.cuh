@@ -147,7 +147,7 @@ __device__ __forceinline__ void tc_ceval(const float* x, float4 nt, float4 nl, f
             float2 r2 = __fmul2_rn(dx, dx);
             r2 = __ffma2_rn(dy, dy, r2);
             r2 = __ffma2_rn(dz, dz, r2);
-            float2 ri = make_float2(tc_green<1, ADJ>(r2.x), tc_green<1, ADJ>(r2.y));
+            float2 ri = make_float2(tc_rsqrt<ADJ>(r2.x), tc_rsqrt<ADJ>(r2.y));
             float2 r = __fmul2_rn(r2, ri);
             r = __ffma2_rn(r, __ffma2_rn(r, __fmul2_rn(ri, tc_f2(-0.5f)), tc_f2(0.5f)), r);
             float2 kr = __fmul2_rn(kap, r);

@@ -279,16 +279,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
                  : "r"(taddr) : "memory");
 }
 
-// kernel value without its constant factor (see Green<>). 3D: the PTX
-// approximate reciprocal square root with subnormals flushed (rsqrt(+inf) = 0
-// gives the masked sources their zero); touching-leaf tiles also zero r^2 <=
-// FLT_MIN (pairs closer than 1.1e-19, coincident points included). 2D: log r^2,
-// zero for r^2 = +inf (masked) and, on touching-leaf tiles, for r^2 = 0.
-template <int KIND, bool ADJ> __device__ __forceinline__ float tc_green(float r2) {
-    if (KIND == 0) {
-        const bool on = r2 < 3.0e38f && (!ADJ || r2 > 0.f);
-        return on ? logf(r2) : 0.f;
-    }
+// 1/r without its constant factor (see Green<>): the PTX approximate reciprocal
+// square root with subnormals flushed (rsqrt(+inf) = 0 gives the masked sources
+// their zero); touching-leaf tiles also zero r^2 <= FLT_MIN (pairs closer than
+// 1.1e-19, coincident points included). 2D: tc_log8.
+template <bool ADJ> __device__ __forceinline__ float tc_rsqrt(float r2) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(r2));
     return (!ADJ || r2 > 1.17549435e-38f) ? y : 0.f;

@@ -168,8 +168,8 @@ __device__ __forceinline__ void tc_eval8(const float* x, float4 nt, float4 nl, f
                 d2[4 * q + 2 * h] = r2.x;
                 d2[4 * q + 2 * h + 1] = r2.y;
             } else {
-                g[4 * q + 2 * h] = tc_green<KIND, ADJ>(r2.x);
-                g[4 * q + 2 * h + 1] = tc_green<KIND, ADJ>(r2.y);
+                g[4 * q + 2 * h] = tc_rsqrt<ADJ>(r2.x);
+                g[4 * q + 2 * h + 1] = tc_rsqrt<ADJ>(r2.y);
             }
         }
     }

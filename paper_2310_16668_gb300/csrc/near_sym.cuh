@@ -16,7 +16,7 @@
 // order: the result does not depend on scheduling, and the items depend on
 // the box pair only.
 // FP64, one right-hand side, near_kernel -> here (whole apply): 3D N = 2^17
-// 42.4 -> 24.8 ms, N = 1,000 924 -> 54 us; 2D N = 16,384 3463 -> 509 us.
+// 42.4 -> 24.8 ms, N = 1,000 924 -> 53 us; 2D N = 16,384 3463 -> 530 us.
 #pragma once
 
 #include "skel_kernels.cuh"

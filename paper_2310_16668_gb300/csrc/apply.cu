@@ -34,6 +34,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <string>
 #include <type_traits>
 
@@ -511,6 +512,7 @@ int run_tc(DevicePlan* dp, DeviceBuffers* b, int nrhs, cudaStream_t st, int& tc_
     t.units = (const TcUnit*)dp->tc_units;
     t.part0 = dp->tc_part0;
     t.parts = dp->tc_parts;
+    t.subnormal = dp->subnormal_r2;
     t.tiles = dp->tc_tiles;
     t.X = (const float4*)b->X;
     t.Xlo = (const float4*)b->Xlo;
@@ -758,6 +760,7 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
         t.units = units;
         t.part0 = nullptr;
         t.parts = nullptr;
+        t.subnormal = dp->subnormal_r2;
         t.tiles = dp->tc_tiles;
         t.X = (const float4*)b->X;
         t.Xlo = (const float4*)b->Xlo;
@@ -1079,6 +1082,8 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
         dp->nrhs_max = nrhs_max;
         dp->top = lay.top;
         dp->L = p.tree.L;
+        // (with a factor of 2 for the rounding of the distances)
+        dp->subnormal_r2 = p.kind == 0 && lay.min_apart < 2.0 * std::sqrt((double)std::numeric_limits<float>::min());
         dp->box_off = upload(lay.box_off, dp->bytes);
         dp->box_n = upload(lay.box_n, dp->bytes);
         dp->box_nslot = upload(lay.box_nslot, dp->bytes);

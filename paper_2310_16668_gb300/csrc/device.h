@@ -48,6 +48,7 @@ struct DevicePlan {
     void* tc_units = nullptr;              // on-the-fly kernel: its CTAs' work (TcUnit)
     int64_t n_units = 0;
     int unit0_item = 0;                    // first item of the first unit (test hook)
+    bool subnormal_r2 = false;             // 2D Laplace: pairs of boxes that do not touch may have subnormal FP32 r^2
     // small plans: tile lists cut over several units, summed per segment
     int64_t* tc_part0 = nullptr;           // per item: its first segment's sums (-1: not cut)
     float* tc_parts = nullptr;

@@ -220,6 +220,7 @@ struct Layout {
     std::vector<uint8_t> entry_slot;    // n_tot: the slot of each entry in its box
     int64_t pairs_direct = 0, pairs_far = 0;
     int64_t pairs_tc = 0;   // kept evaluations inside tensor-core items
+    double min_apart = 0.0; // side of the finest boxes: pairs not flagged TASK_ADJ are at least this far apart
 };
 
 void build_layout(const Plan& p, Layout& lay);

@@ -22,6 +22,7 @@
 // Tasks between two touching leaves are flagged TASK_ADJ: only they can hold
 // arbitrarily close (or coincident) pairs.
 #include <algorithm>
+#include <cmath>
 #include <numeric>
 
 #include "host.h"
@@ -45,6 +46,7 @@ void build_layout(const Plan& p, Layout& lay) {
     const int dim = t.dim;
     const int64_t nb = t.nb;
     lay.top = t.L >= 1 ? 1 : 0;
+    lay.min_apart = std::ldexp(t.side, -t.L);
 
     // ---- entry space ----------------------------------------------------
     lay.box_off.assign(nb, -1);
@@ -562,6 +564,7 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
         m.pairs_direct += l.pairs_direct;
         m.pairs_far += l.pairs_far;
         m.pairs_tc += l.pairs_tc;
+        m.min_apart = s == 0 ? l.min_apart : std::min(m.min_apart, l.min_apart);
     }
     if (!sym) {
         m.sym_items.clear();

@@ -102,6 +102,7 @@ struct TcArgs {
     const TcUnit* units;                       // on-the-fly kernel: the CTAs' work
     const int64_t* part0;                      // per item: its first segment in parts, -1 if it is not cut
     float* parts;                              // sums of the segments of cut items, 128 rows x 32 (null: none)
+    bool subnormal;                            // 2D: r^2 may be subnormal between boxes that do not touch
     const SrcTile* tiles;                      // item i's tiles: [list_lo, list_hi) of this array
     const float4* X;
     const float4* Xlo;

@@ -80,9 +80,10 @@ static_assert(sizeof(TcNearShared) <= kNearSmemRequest, "shared memory plan");
 // P of degree 7 fitted to the series (relative error 6e-9), ln 2 as a sum of
 // two floats the first of which has 9 significant bits: within 0.9 ulp, half
 // the instructions of logf because two values share each. on: 1, or 0 for a row
-// that keeps none of these sources. ADJ: 0 for x = 0, and logf for subnormal x.
+// that keeps none of these sources. ADJ: subnormal x (whose exponent field says
+// nothing) go to logf; 0 for x = 0 if the leaves touch.
 template <bool ADJ>
-__device__ __forceinline__ void tc_log8(const float* r2, float on, float* g) {
+__device__ __forceinline__ void tc_log8(const float* r2, float on, bool touch, float* g) {
     auto f2 = [](float v) { return make_float2(v, v); };
     const float2 on2 = f2(on);
 #pragma unroll
@@ -120,7 +121,7 @@ __device__ __forceinline__ void tc_log8(const float* r2, float on, float* g) {
         if (__any_sync(0xffffffffu, lo < 1.17549435e-38f)) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                if (r2[j] < 1.17549435e-38f) g[j] = r2[j] > 0.f ? on * logf(r2[j]) : 0.f;
+                if (r2[j] < 1.17549435e-38f) g[j] = !touch || r2[j] > 0.f ? on * logf(r2[j]) : 0.f;
             __syncwarp();
         }
     }
@@ -128,9 +129,10 @@ __device__ __forceinline__ void tc_log8(const float* r2, float on, float* g) {
 
 // 8 sources (coordinates at x: 32 floats per axis; lo parts 96 floats on)
 // against this thread's target, two sources per paired FP32 instruction: the
-// kernel values in g, not masked. nt, nl: the negated target.
+// kernel values in g, not masked. nt, nl: the negated target. touch: of two
+// touching leaves.
 template <int KIND, bool ADJ>
-__device__ __forceinline__ void tc_eval8(const float* x, float4 nt, float4 nl, float* g) {
+__device__ __forceinline__ void tc_eval8(const float* x, float4 nt, float4 nl, bool touch, float* g) {
     constexpr int AX = 32, LO = 96;
     const float2 ntx = make_float2(nt.x, nt.x), nty = make_float2(nt.y, nt.y), ntz = make_float2(nt.z, nt.z);
     float d2[KIND == 0 ? 8 : 1];
@@ -173,7 +175,7 @@ __device__ __forceinline__ void tc_eval8(const float* x, float4 nt, float4 nl, f
             }
         }
     }
-    if constexpr (KIND == 0) tc_log8<ADJ>(d2, nt.x < kFar ? 1.f : 0.f, g);
+    if constexpr (KIND == 0) tc_log8<ADJ>(d2, nt.x < kFar ? 1.f : 0.f, touch, g);
 }
 
 // Veltkamp's split of 8 values into TF32 hi and lo: hi = t - (t - g) with
@@ -355,7 +357,12 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
             if (ti == 0) ok &= mbar_wait(sm_addr(&S.full[ring + s]), ph, a.wait_ns);
             const SrcTile& tl = st.tile[ti];
             const float* xs = st.chunk[ti] + 2048;
-            const bool adj = (tl.flags & TASK_ADJ) != 0;
+            // touching leaves take the form with lo parts and guards, and so do
+            // the other boxes of a 2D plan so small that their r^2 may be
+            // subnormal (guards in the other form cost every 2D plan 13% of
+            // this kernel: N = 65,536 218 -> 246 us)
+            const bool touch = (tl.flags & TASK_ADJ) != 0;
+            const bool adj = touch || (KIND == 0 && a.subnormal);
             uint32_t all = tl.cnt >= 32 ? 0xFFFFFFFFu : (1u << (tl.cnt & 31)) - 1u;
             if (SPLIT) all = all >> (16 * g) & 0xFFFFu;
             const TcNearTile ta = tc_near_tile<REC>(rw, tl, all, adj, SPLIT ? 16 * g : 0);
@@ -400,7 +407,7 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
                             float4 at = ta.nt;
                             bool cut = false;
                             if constexpr (decltype(CUT)::value) cut = tc_near_cut(ta, all, q, at);
-                            tc_eval8<KIND, decltype(ADJ)::value>(xq, at, ta.nl, gv);
+                            tc_eval8<KIND, decltype(ADJ)::value>(xq, at, ta.nl, touch, gv);
                             if constexpr (REC == kRecSym) {
                                 // this row's block of the tile, if this tile records it
                                 // (stored as this row chunk x the tile's chunk)

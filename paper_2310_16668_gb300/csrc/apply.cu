@@ -314,14 +314,19 @@ void ud_narrow_launch(const DevicePlan* dp, int l, int nrhs, const S* T, S* X, b
     else if constexpr (sizeof(S) <= 8) ud_narrow_launch_rt<S, DOWN, 8>(dp, l, nrhs, T, X, conj_op, st);
 }
 
+// few right-hand sides: a row per lane instead of a column (every launch shape
+// of the other kernels puts 32 columns on the lanes)
+template <class S>
+constexpr bool ud_narrow(int nrhs) {
+    return nrhs <= (sizeof(S) <= 8 ? kUnMaxRhs : 4);
+}
+
 // one level of the upward or downward pass; warps = 0: the level's setting
 // (autotuned for FP32, else the default rule)
 template <class S>
 void up_down(bool down, const DevicePlan* dp, int l, const S* T, S* X, int nrhs, bool conj_op, cudaStream_t st,
              int warps = 0) {
-    // few right-hand sides: a row per lane instead of a column (every launch
-    // shape below puts 32 columns on the lanes)
-    if (nrhs <= (sizeof(S) <= 8 ? kUnMaxRhs : 4)) {
+    if (ud_narrow<S>(nrhs)) {
         down ? ud_narrow_launch<S, true>(dp, l, nrhs, T, X, conj_op, st)
              : ud_narrow_launch<S, false>(dp, l, nrhs, T, X, conj_op, st);
         return;
@@ -1382,10 +1387,13 @@ TuneReport device_autotune(DevicePlan* dp, int nrhs, bool allow_store, void* str
             return (double)ms / reps;
         };
         // 1. up/down launch shape per level: warps per CTA (every choice
-        //    adds the same partial sums in the same order)
-        const int nl = (int)dp->up_level_ptr.size() - 1;
-        dp->ud_warps_up.assign(std::max(nl, 0), 0);
-        dp->ud_warps_down.assign(std::max(nl, 0), 0);
+        //    adds the same partial sums in the same order); few right-hand
+        //    sides have one shape, and the settings of the others stay
+        const int nl = ud_narrow<float>(nrhs) ? 0 : (int)dp->up_level_ptr.size() - 1;
+        if (nl > 0) {
+            dp->ud_warps_up.assign(nl, 0);
+            dp->ud_warps_down.assign(nl, 0);
+        }
         for (int l = 2; l <= dp->L && l < nl; ++l) {
             if (dp->up_level_ptr[l + 1] == dp->up_level_ptr[l]) continue;
             for (int down = 0; down < 2; ++down) {

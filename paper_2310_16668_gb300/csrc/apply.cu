@@ -119,6 +119,12 @@ T* upload(const std::vector<T>& v, int64_t& bytes) {
 // 1.22 ms against 1.12).
 constexpr int kSymMaxRhs = 4;
 int sym_columns(int nrhs) { return nrhs == 1 ? 1 : 2; }
+// Slots of a batch of symmetric translations, at most: 537 MB per FP64 column
+// (a 3D plan of N = 2^20 has 13.9 million slots, 3.6 GB). A batch ends in a wave
+// that is not full, about 0.1 ms: N = 2^20, one column, all slots at once 255.9 ms,
+// batches of 2^21 256.5, 2^20 257.2, 2^19 258.3; N = 2^17 (one batch of 2^21) 24.8,
+// 24.8, 24.85, 24.95.
+constexpr int64_t kSymBatchSlots = (int64_t)1 << 21;
 template <class Real>
 bool use_sym(const DevicePlan* dp, int nrhs) {
     return sizeof(Real) == 8 && dp->n_sym > 0 && nrhs <= kSymMaxRhs;
@@ -431,14 +437,21 @@ NearArgs<Real, CPLX> near_args(DevicePlan* dp, DeviceBuffers* b, const WorkItem*
 }
 
 template <int KIND, int RT>
-int sym_pass(const SymArgs<cplx_kind(KIND)>& a, const DevicePlan* dp, cudaStream_t st) {
+int sym_pass(SymArgs<cplx_kind(KIND)> a, const DevicePlan* dp, cudaStream_t st) {
     using S = typename Scal<double, cplx_kind(KIND)>::T;
-    sym_kernel<KIND, RT><<<ceil_div(dp->n_sym, kSymWarps), kSymWarps * 32, 0, st>>>(a);
-    CUDA_CHECK(cudaGetLastError());
-    sym_reduce_kernel<S, RT><<<ceil_div(dp->n_chunks * 32, 256), 256, 0, st>>>(
-        dp->sym_ptr, dp->sym_idx, dp->chunk_start, dp->chunk_cnt, dp->n_chunks, a.part, (S*)dp->p64->U, a.nrhs, a.r0);
-    CUDA_CHECK(cudaGetLastError());
-    return 2;
+    int launches = 0;
+    for (size_t b = 0; b + 1 < dp->sym_item_ptr.size(); ++b) {
+        a.items = dp->sym_items + dp->sym_item_ptr[b];
+        a.n_items = dp->sym_item_ptr[b + 1] - dp->sym_item_ptr[b];
+        sym_kernel<KIND, RT><<<ceil_div(a.n_items, kSymWarps), kSymWarps * 32, 0, st>>>(a);
+        CUDA_CHECK(cudaGetLastError());
+        const int64_t r0 = dp->sym_run_ptr[b], n = dp->sym_run_ptr[b + 1] - r0;
+        sym_reduce_kernel<S, RT><<<ceil_div(n * 32, 256), 256, 0, st>>>(
+            dp->sym_runs + r0, n, dp->sym_idx, dp->chunk_start, dp->chunk_cnt, a.part, (S*)dp->p64->U, a.nrhs, a.r0);
+        CUDA_CHECK(cudaGetLastError());
+        launches += 2;
+    }
+    return launches;
 }
 
 template <int KIND>
@@ -446,8 +459,6 @@ int run_sym_kind(const DevicePlan* dp, int nrhs, cudaStream_t st) {
     using S = typename Scal<double, cplx_kind(KIND)>::T;
     const DeviceBuffers* b = dp->p64;
     SymArgs<cplx_kind(KIND)> a;
-    a.items = dp->sym_items;
-    a.n_items = dp->n_sym;
     a.chunk_start = dp->chunk_start;
     a.chunk_cnt = dp->chunk_cnt;
     a.entry_slot = dp->entry_slot;
@@ -1215,11 +1226,14 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
         dp->chunk_cnt = upload(lay.chunk_cnt, dp->bytes);
         dp->n_chunks = (int64_t)lay.chunk_start.size();
         dp->n_sym = (int64_t)lay.sym_items.size();
-        dp->sym_slots = lay.sym_slots;
         if (dp->n_sym > 0) {
-            dp->sym_items = upload(lay.sym_items, dp->bytes);
-            dp->sym_ptr = upload(lay.sym_ptr, dp->bytes);
-            dp->sym_idx = upload(lay.sym_idx, dp->bytes);
+            const SymPlan s = make_sym_plan(lay, kSymBatchSlots);
+            dp->sym_slots = s.slots;
+            dp->sym_items = upload(s.items, dp->bytes);
+            dp->sym_runs = upload(s.runs, dp->bytes);
+            dp->sym_idx = upload(s.idx, dp->bytes);
+            dp->sym_item_ptr = s.item_ptr;
+            dp->sym_run_ptr = s.run_ptr;
             dp->entry_slot = upload(lay.entry_slot, dp->bytes);
             if (dp->kind == 0) dp->logtab = upload(log_table(), dp->bytes);
         }
@@ -1280,7 +1294,7 @@ void device_plan_destroy(DevicePlan* dp) {
     cudaSetDevice(dp->device);
     void* ptrs[] = {dp->box_off, dp->box_n, dp->box_nslot, dp->slot_start, dp->pos, dp->eop, dp->eop2, dp->up, dp->task_src, dp->task_mask, dp->task_flags, dp->items,
                     dp->part_ptr, dp->part_idx, dp->stage_in, dp->stage_out, dp->mix_items, dp->tc_tiles,
-                    dp->tc_items, dp->sym_items, dp->sym_ptr, dp->sym_idx, dp->entry_slot, dp->logtab, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
+                    dp->tc_items, dp->sym_items, dp->sym_runs, dp->sym_idx, dp->entry_slot, dp->logtab, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
                     dp->tc_part_ptr, dp->tc_part_idx, dp->status,
                     dp->chunk_start, dp->chunk_cnt, dp->chunk_center, dp->tc_b, dp->tc_a, dp->tc_abase,
                     dp->tc_qmask, dp->tc_refs, dp->tc_isym, dp->ud_items_up, dp->ud_items_down,

@@ -57,11 +57,12 @@ struct DevicePlan {
     int64_t tc_n_slots = 0;
     int64_t* tc_part_ptr = nullptr;        // per entry: its partial sums (tensor-core mode)
     int64_t* tc_part_idx = nullptr;
-    // symmetric CUDA-core translations (n_sym = 0: none)
+    // symmetric CUDA-core translations (n_sym = 0: none), in batches (SymPlan)
     SymItem* sym_items = nullptr;
-    int64_t n_sym = 0, sym_slots = 0;
-    int64_t* sym_ptr = nullptr;            // per chunk: its slots
+    int64_t n_sym = 0, sym_slots = 0;      // items; slots of the largest batch
+    SymRun* sym_runs = nullptr;
     int32_t* sym_idx = nullptr;
+    std::vector<int64_t> sym_item_ptr, sym_run_ptr;
     uint8_t* entry_slot = nullptr;
     double* logtab = nullptr;              // 2D Laplace: table of log_f64
     int64_t* chunk_start = nullptr;        // source chunks (32 entries of one box)

@@ -128,8 +128,8 @@ struct WorkItem {                       // one warp: 32 targets x a task range
 };
 
 // One unordered pair (target chunk, source chunks of one box) of the symmetric
-// CUDA-core translations: slot `slot` of 32 rows takes the target chunk's sums,
-// slot + 1 + k those of source chunk schunk + k.
+// CUDA-core translations: slot `slot` of 32 rows (of its batch, see SymPlan)
+// takes the target chunk's sums, slot + 1 + k those of source chunk schunk + k.
 struct SymItem {                        // 32 bytes
     uint64_t mask;                      // bit (c*8 + c'): skip target slot c x source slot c'
     int32_t tchunk, schunk;             // first source chunk
@@ -211,12 +211,10 @@ struct Layout {
     std::vector<int64_t> chunk_start;   // first entry of each chunk
     std::vector<int32_t> chunk_cnt;     // entries in it (1..32)
     std::vector<float> chunk_center;    // 4 per chunk: its box's centre (FP32), 0
-    // symmetric CUDA-core translations: items, their slots, and per chunk the
-    // slots that add up to its entries (empty if the tasks are not symmetric)
+    // symmetric CUDA-core translations: items (without their slots) and the
+    // slots of all (empty if the tasks are not symmetric)
     std::vector<SymItem> sym_items;
     int64_t sym_slots = 0;
-    std::vector<int64_t> sym_ptr;       // chunks + 1
-    std::vector<int32_t> sym_idx;
     std::vector<uint8_t> entry_slot;    // n_tot: the slot of each entry in its box
     int64_t pairs_direct = 0, pairs_far = 0;
     int64_t pairs_tc = 0;   // kept evaluations inside tensor-core items
@@ -224,6 +222,23 @@ struct Layout {
 };
 
 void build_layout(const Plan& p, Layout& lay);
+
+// The symmetric translations in batches that share one buffer of slots: batch
+// i is items [item_ptr[i], item_ptr[i+1]) and then runs [run_ptr[i],
+// run_ptr[i+1]), each of which adds its slots (idx[at .. at + n)) to a chunk.
+struct SymRun {                         // 16 bytes
+    int64_t at;
+    int32_t chunk;                      // ~chunk: not its first run (adds to U, the first overwrites it)
+    int32_t n;
+};
+struct SymPlan {
+    std::vector<SymItem> items;
+    std::vector<SymRun> runs;
+    std::vector<int32_t> idx;
+    std::vector<int64_t> item_ptr, run_ptr;
+    int64_t slots = 0;                  // of the largest batch
+};
+SymPlan make_sym_plan(const Layout& lay, int64_t max_slots);
 
 // class of a tensor-core item's tile-list length (lengths within a factor
 // 1.25 share a class); items run longest class first

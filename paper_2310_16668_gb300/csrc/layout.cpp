@@ -392,8 +392,6 @@ void build_layout(const Plan& p, Layout& lay) {
     }
     lay.sym_items.clear();
     lay.sym_slots = 0;
-    lay.sym_ptr.assign(lay.chunk_start.size() + 1, 0);
-    lay.sym_idx.clear();
     auto slots_of = [&](int64_t chunk) {
         unsigned m = 0;
         for (int32_t e = 0; e < lay.chunk_cnt[chunk]; ++e) m |= 1u << lay.entry_slot[lay.chunk_start[chunk] + e];
@@ -402,7 +400,6 @@ void build_layout(const Plan& p, Layout& lay) {
     std::vector<uint8_t> chunk_slots(lay.chunk_start.size());
     for (size_t c = 0; c < chunk_slots.size(); ++c) chunk_slots[c] = (uint8_t)slots_of((int64_t)c);
     int64_t up_pairs = 0, down_pairs = 0;                   // kept pairs of tasks to higher / lower boxes
-    std::vector<std::pair<int32_t, int32_t>> owner;         // (chunk, slot) in slot order
     for (int64_t b = 0; b < nb; ++b) {
         if (lay.box_off[b] < 0) continue;
         const int64_t tc0 = lay.box_chunk0[b], ntc = (lay.box_n[b] + kTcK - 1) / kTcK;
@@ -429,10 +426,6 @@ void build_layout(const Plan& p, Layout& lay) {
                                 (chunk_slots[sc0 + j] & ~(unsigned)(mask >> (8 * c)) & 0xFFu))
                                 any = true;
                     if (it.nsrc > 0 && (!any || it.nsrc == per)) {
-                        it.slot = (int32_t)lay.sym_slots;
-                        owner.push_back({it.tchunk, it.slot});
-                        for (int k = 0; k < it.nsrc; ++k)
-                            if (it.schunk + k != it.tchunk) owner.push_back({it.schunk + k, it.slot + 1 + k});
                         lay.sym_slots += 1 + it.nsrc;
                         if (lay.sym_slots > INT32_MAX - 16) throw Error(-1, "too many translations");
                         lay.sym_items.push_back(it);
@@ -453,13 +446,62 @@ void build_layout(const Plan& p, Layout& lay) {
     if (up_pairs != down_pairs) {
         lay.sym_items.clear();
         lay.sym_slots = 0;
-    } else {
-        for (const auto& o : owner) lay.sym_ptr[o.first + 1]++;
-        for (size_t c = 0; c + 1 < lay.sym_ptr.size(); ++c) lay.sym_ptr[c + 1] += lay.sym_ptr[c];
-        lay.sym_idx.resize(owner.size());
-        std::vector<int64_t> at(lay.sym_ptr.begin(), lay.sym_ptr.end() - 1);
-        for (const auto& o : owner) lay.sym_idx[at[o.first]++] = o.second;
     }
+}
+
+SymPlan make_sym_plan(const Layout& lay, int64_t max_slots) {
+    SymPlan p;
+    p.items = lay.sym_items;
+    const int64_t n = (int64_t)p.items.size(), nch = (int64_t)lay.chunk_start.size();
+    // batches of nearly the same number of slots
+    const int64_t share = max_slots - 8;                    // an item has at most 5 slots
+    const int64_t nbatch = std::max<int64_t>(1, (lay.sym_slots + share - 1) / share);
+    const int64_t target = (lay.sym_slots + nbatch - 1) / nbatch;
+    p.item_ptr.push_back(0);
+    int64_t cur = 0;
+    for (int64_t i = 0; i < n; ++i) {
+        if (cur >= target) {
+            p.item_ptr.push_back(i);
+            cur = 0;
+        }
+        p.items[i].slot = (int32_t)cur;
+        cur += 1 + p.items[i].nsrc;
+        p.slots = std::max(p.slots, cur);
+    }
+    p.item_ptr.push_back(n);
+    // per batch the slots of each chunk, in the order of the items
+    auto owners = [&](const SymItem& it, auto&& f) {
+        f(it.tchunk, it.slot);
+        for (int k = 0; k < it.nsrc; ++k)
+            if (it.schunk + k != it.tchunk) f(it.schunk + k, it.slot + 1 + k);
+    };
+    std::vector<int64_t> at(nch);
+    std::vector<int32_t> cnt(nch);
+    std::vector<char> seen(nch, 0);
+    p.run_ptr.push_back(0);
+    for (size_t b = 0; b + 1 < p.item_ptr.size(); ++b) {
+        std::fill(cnt.begin(), cnt.end(), 0);
+        for (int64_t i = p.item_ptr[b]; i < p.item_ptr[b + 1]; ++i)
+            owners(p.items[i], [&](int32_t c, int32_t) { ++cnt[c]; });
+        int64_t end = (int64_t)p.idx.size();
+        const bool last = b + 2 == p.item_ptr.size();
+        for (int64_t c = 0; c < nch; ++c) {
+            // (a chunk without any slot still has its rows of U set to zero)
+            if (cnt[c] == 0 && !(last && !seen[c])) continue;
+            p.runs.push_back(SymRun{end, (int32_t)(seen[c] ? ~c : c), cnt[c]});
+            seen[c] = 1;
+            at[c] = end;
+            end += cnt[c];
+        }
+        p.run_ptr.push_back((int64_t)p.runs.size());
+        p.idx.resize(end);
+        for (int64_t i = p.item_ptr[b]; i < p.item_ptr[b + 1]; ++i)
+            owners(p.items[i], [&](int32_t c, int32_t slot) { p.idx[at[c]++] = slot; });
+        // a batch runs its longest items first: its last wave is then short
+        std::stable_sort(p.items.begin() + p.item_ptr[b], p.items.begin() + p.item_ptr[b + 1],
+                         [](const SymItem& x, const SymItem& y) { return x.nsrc > y.nsrc; });
+    }
+    return p;
 }
 
 }  // namespace skel
@@ -546,13 +588,8 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
         for (SymItem it : l.sym_items) {
             it.tchunk = (int32_t)(it.tchunk + c0[s]);
             it.schunk = (int32_t)(it.schunk + c0[s]);
-            it.slot = (int32_t)(it.slot + m.sym_slots);
             m.sym_items.push_back(it);
         }
-        if (m.sym_ptr.empty()) m.sym_ptr.push_back(0);
-        for (size_t c = 1; c < l.sym_ptr.size(); ++c)
-            m.sym_ptr.push_back((int64_t)m.sym_idx.size() + l.sym_ptr[c]);
-        for (int32_t v : l.sym_idx) m.sym_idx.push_back((int32_t)(v + m.sym_slots));
         m.sym_slots += l.sym_slots;
         sym &= l.sym_slots > 0;
         if (m.sym_slots > INT32_MAX) throw Error(-1, "merged plan too large (more than 2^31 partial sums)");

@@ -14,7 +14,8 @@
 // to lane (one shuffle per step) and end at their own lane. Both sides' sums
 // go to slots of 32 rows, which sym_reduce_kernel adds per chunk in a fixed
 // order: the result does not depend on scheduling, and the items depend on
-// the box pair only.
+// the box pair only. The items run in batches that share one buffer of slots
+// (kSymBatchSlots), so that its size is bounded.
 // FP64, one right-hand side, near_kernel -> here (whole apply): 3D N = 2^17
 // 42.4 -> 24.8 ms, N = 1,000 924 -> 53 us; 2D N = 16,384 3463 -> 530 us.
 #pragma once
@@ -172,21 +173,29 @@ __global__ void __launch_bounds__(kSymWarps * 32) sym_kernel(const SymArgs<cplx_
     for (int r = 0; r < RT; ++r) a.part[((int64_t)it.slot * 32 + lane) * RT + r] = scale * at[r];
 }
 
-// U of every chunk: the sum of its slots, in order. A warp per chunk, lane =
-// entry; eight slots' loads in flight. Bound: HBM (the slots).
+// The sums of a batch's slots, in order, to U. A warp per run (a chunk's slots of
+// this batch), lane = entry; eight slots' loads in flight. The first run of a
+// chunk overwrites its rows of U, the others go on from them, so the sum does
+// not depend on how the items are cut into batches. Bound: HBM (the slots).
 template <class S, int RT>
-__global__ void __launch_bounds__(256) sym_reduce_kernel(const int64_t* __restrict__ ptr, const int32_t* __restrict__ idx,
+__global__ void __launch_bounds__(256) sym_reduce_kernel(const SymRun* __restrict__ runs, int64_t n_runs,
+                                                         const int32_t* __restrict__ idx,
                                                          const int64_t* __restrict__ chunk_start,
-                                                         const int32_t* __restrict__ chunk_cnt, int64_t n_chunks,
+                                                         const int32_t* __restrict__ chunk_cnt,
                                                          const S* __restrict__ part, S* __restrict__ U, int nrhs, int r0) {
-    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (c >= n_chunks) return;
+    if (id >= n_runs) return;
+    const SymRun run = runs[id];
+    const bool first = run.chunk >= 0;
+    const int c = first ? run.chunk : ~run.chunk;
+    const bool valid = lane < chunk_cnt[c];
+    S* u = U + (chunk_start[c] + lane) * nrhs + r0;
     S sum[RT];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) sum[r] = zero<S>();
-    const int64_t p1 = ptr[c + 1];
-    for (int64_t p = ptr[c]; p < p1; p += 8) {
+    for (int r = 0; r < RT; ++r) sum[r] = !first && valid && r0 + r < nrhs ? u[r] : zero<S>();
+    const int64_t p1 = run.at + run.n;
+    for (int64_t p = run.at; p < p1; p += 8) {
         S v[8][RT];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -201,10 +210,10 @@ __global__ void __launch_bounds__(256) sym_reduce_kernel(const int64_t* __restri
 #pragma unroll
                 for (int r = 0; r < RT; ++r) sum[r] += v[q][r];
     }
-    if (lane < chunk_cnt[c]) {
+    if (valid) {
 #pragma unroll
         for (int r = 0; r < RT; ++r)
-            if (r0 + r < nrhs) U[(chunk_start[c] + lane) * nrhs + r0 + r] = sum[r];
+            if (r0 + r < nrhs) u[r] = sum[r];
     }
 }
 

@@ -427,7 +427,6 @@ void build_layout(const Plan& p, Layout& lay) {
                                 any = true;
                     if (it.nsrc > 0 && (!any || it.nsrc == per)) {
                         lay.sym_slots += 1 + it.nsrc;
-                        if (lay.sym_slots > INT32_MAX - 16) throw Error(-1, "too many translations");
                         lay.sym_items.push_back(it);
                         it.nsrc = 0;
                     }
@@ -592,7 +591,6 @@ void merge_layouts(const std::vector<const Layout*>& ls, const std::vector<int64
         }
         m.sym_slots += l.sym_slots;
         sym &= l.sym_slots > 0;
-        if (m.sym_slots > INT32_MAX) throw Error(-1, "merged plan too large (more than 2^31 partial sums)");
         m.entry_slot.insert(m.entry_slot.end(), l.entry_slot.begin(), l.entry_slot.end());
         for (int64_t v : l.box_chunk0) m.box_chunk0.push_back(v < 0 ? -1 : v + c0[s]);
         for (int64_t v : l.chunk_start) m.chunk_start.push_back(v + e0[s]);

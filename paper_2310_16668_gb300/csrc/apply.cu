@@ -34,9 +34,11 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <future>
 #include <limits>
 #include <string>
 #include <type_traits>
+#include <utility>
 
 #include "device.h"
 #include "skel_kernels.cuh"
@@ -111,6 +113,33 @@ T* upload(const std::vector<T>& v, int64_t& bytes) {
     return p;
 }
 
+// several arrays in one allocation and, if they are small, by one copy (the
+// device part of a plan of 1,000 points takes 0.4 ms, an allocation or a copy
+// about 0.01 of it); returns the allocation
+template <class... T>
+void* upload_all(int64_t& bytes, std::pair<const std::vector<T>&, T**>... arrays) {
+    auto size = [](const auto& v) { return (v.size() * sizeof(v[0]) + 255) / 256 * 256; };
+    const size_t total = (size(arrays.first) + ...);
+    char* base = dalloc<char>(total, bytes);
+    size_t at = 0;
+    try {
+        std::vector<char> joined(total <= (size_t)1 << 20 ? total : 0);
+        auto put = [&](const auto& v, auto** p) {
+            *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + at);
+            const size_t n = v.size() * sizeof(v[0]);
+            if (n > 0 && !joined.empty()) std::memcpy(joined.data() + at, v.data(), n);
+            else if (n > 0) CUDA_CHECK(cudaMemcpy(base + at, v.data(), n, cudaMemcpyHostToDevice));
+            at += size(v);
+        };
+        (put(arrays.first, arrays.second), ...);
+        if (!joined.empty()) CUDA_CHECK(cudaMemcpy(base, joined.data(), total, cudaMemcpyHostToDevice));
+    } catch (...) {
+        cudaFree(base);
+        throw;
+    }
+    return base;
+}
+
 // Right-hand sides per pass of the symmetric translations: 6.5 and 7.5 FP64
 // operations an interaction (of 3D Laplace) for 1 and 2 columns, against 12 in
 // near_kernel for one and 19 for a pass of up to 8. Two passes of two columns
@@ -131,7 +160,7 @@ bool use_sym(const DevicePlan* dp, int nrhs) {
 }
 
 // the table of log_f64: 1/c, and log c as a multiple of 2^-40 and the rest
-std::vector<double> log_table() {
+std::vector<double> make_log_table() {
     std::vector<double> t(3 * kLogTab);
     auto value = [](int64_t bits) {
         double v;
@@ -147,6 +176,10 @@ std::vector<double> log_table() {
         t[kLogTab + i] = std::ldexp(std::nearbyint(std::ldexp((double)c, 40)), -40);
         t[2 * kLogTab + i] = (double)(c - (long double)t[kLogTab + i]);
     }
+    return t;
+}
+const std::vector<double>& log_table() {
+    static const std::vector<double> t = make_log_table();
     return t;
 }
 
@@ -1085,6 +1118,8 @@ void build_ud_items(bool down, const std::vector<UpBox>& up, const std::vector<i
 
 DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, int store_tiles, int store_stages,
                                bool updown_tc) {
+    // (beside the uploads)
+    std::future<SymPlan> sym = std::async(host_task(lay), [&lay] { return make_sym_plan(lay, kSymBatchSlots); });
     DevicePlan* dp = new DevicePlan();
     dp->tcs_stages = store_stages == 8 || store_stages == 5 ? store_stages : 4;
     try {
@@ -1214,29 +1249,20 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
             const Units u = make_units(lay.tc_items, dp->dim);
             dp->n_units = (int64_t)u.units.size();
             dp->unit0_item = u.units[0].a;
-            dp->tc_units = upload(u.units, dp->bytes);
             dp->n_split = (int64_t)u.split.size();
+            TcUnit* units = nullptr;
+            int64_t* part0 = nullptr;
+            dp->unit_block = upload_all<TcUnit, int64_t, int32_t>(dp->bytes, {u.units, &units}, {u.part0, &part0},
+                                                                  {u.split, &dp->tc_split});
+            dp->tc_units = units;
             if (dp->n_split > 0) {
-                dp->tc_part0 = upload(u.part0, dp->bytes);
-                dp->tc_split = upload(u.split, dp->bytes);
+                dp->tc_part0 = part0;
                 dp->tc_parts = dalloc<float>((size_t)u.segments * kTcRows * kTcN, dp->bytes);
             }
         }
         dp->chunk_start = upload(lay.chunk_start, dp->bytes);
         dp->chunk_cnt = upload(lay.chunk_cnt, dp->bytes);
         dp->n_chunks = (int64_t)lay.chunk_start.size();
-        dp->n_sym = (int64_t)lay.sym_items.size();
-        if (dp->n_sym > 0) {
-            const SymPlan s = make_sym_plan(lay, kSymBatchSlots);
-            dp->sym_slots = s.slots;
-            dp->sym_items = upload(s.items, dp->bytes);
-            dp->sym_runs = upload(s.runs, dp->bytes);
-            dp->sym_idx = upload(s.idx, dp->bytes);
-            dp->sym_item_ptr = s.item_ptr;
-            dp->sym_run_ptr = s.run_ptr;
-            dp->entry_slot = upload(lay.entry_slot, dp->bytes);
-            if (dp->kind == 0) dp->logtab = upload(log_table(), dp->bytes);
-        }
         if (dp->n_tc > 0 && (!dp->cplx || dp->kind == 2)) {
             dp->chunk_center = upload(lay.chunk_center, dp->bytes);
             dp->tc_b = dalloc<float>((size_t)dp->n_chunks * (dp->cplx ? kChunkFloatsC : kChunkFloats), dp->bytes);
@@ -1246,10 +1272,20 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
         dp->tc_part_idx = upload(lay.tc_part_idx, dp->bytes);
         dp->status = dalloc<int>(1, dp->bytes);
         CUDA_CHECK(cudaMemset(dp->status, 0, sizeof(int)));
-        dp->p64 = new DeviceBuffers();
-        make_buffers<double>(dp, lay, dp->p64);
         dp->p32 = new DeviceBuffers();
         make_buffers<float>(dp, lay, dp->p32);
+        dp->n_sym = (int64_t)lay.sym_items.size();
+        if (dp->n_sym > 0) {
+            const SymPlan s = sym.get();
+            dp->sym_slots = s.slots;
+            dp->sym_item_ptr = s.item_ptr;
+            dp->sym_run_ptr = s.run_ptr;
+            dp->sym_block = upload_all<SymItem, SymRun, int32_t, uint8_t, double>(
+                dp->bytes, {s.items, &dp->sym_items}, {s.runs, &dp->sym_runs}, {s.idx, &dp->sym_idx},
+                {lay.entry_slot, &dp->entry_slot}, {dp->kind == 0 ? log_table() : std::vector<double>(), &dp->logtab});
+        }
+        dp->p64 = new DeviceBuffers();
+        make_buffers<double>(dp, lay, dp->p64);
         if (dp->n_tc > 0 && !dp->cplx) {
             dp->n_tc_tiles = (int64_t)lay.tc_tiles.size();
             for (const TcItem& it : lay.tc_items)
@@ -1294,7 +1330,7 @@ void device_plan_destroy(DevicePlan* dp) {
     cudaSetDevice(dp->device);
     void* ptrs[] = {dp->box_off, dp->box_n, dp->box_nslot, dp->slot_start, dp->pos, dp->eop, dp->eop2, dp->up, dp->task_src, dp->task_mask, dp->task_flags, dp->items,
                     dp->part_ptr, dp->part_idx, dp->stage_in, dp->stage_out, dp->mix_items, dp->tc_tiles,
-                    dp->tc_items, dp->sym_items, dp->sym_runs, dp->sym_idx, dp->entry_slot, dp->logtab, dp->tc_units, dp->tc_part0, dp->tc_parts, dp->tc_split,
+                    dp->tc_items, dp->sym_block, dp->unit_block, dp->tc_parts,
                     dp->tc_part_ptr, dp->tc_part_idx, dp->status,
                     dp->chunk_start, dp->chunk_cnt, dp->chunk_center, dp->tc_b, dp->tc_a, dp->tc_abase,
                     dp->tc_qmask, dp->tc_refs, dp->tc_isym, dp->ud_items_up, dp->ud_items_down,

@@ -83,6 +83,7 @@ void finalize(skel_plan* h, const skel_options* opts) {
     h->host_only = opts && opts->host_only;
     double t0 = now();
     skel::Layout lay;
+    lay.threads = opts && opts->num_threads > 0 ? opts->num_threads : 0;
     skel::build_layout(h->plan, lay);
     h->n_items = (int64_t)lay.items.size();
     h->pairs_direct = lay.pairs_direct;
@@ -409,6 +410,7 @@ int skel_merge(const skel_handle* hs, int nsets, const skel_options* opts, skel_
         const skel::Plan& P0 = hs[0]->plan;
         skel::Layout m;
         skel::merge_layouts(lp, np, nb, P0.sk.cplx ? 2 : 1, m);
+        m.threads = opts && opts->num_threads > 0 ? opts->num_threads : 0;
         lays.clear();
         skel_plan* h = new skel_plan();
         try {

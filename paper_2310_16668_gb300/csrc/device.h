@@ -45,6 +45,7 @@ struct DevicePlan {
     SrcTile* tc_tiles = nullptr;
     TcItem* tc_items = nullptr;
     int64_t n_tc = 0;
+    void* unit_block = nullptr;            // the allocation of tc_units, tc_part0 and tc_split
     void* tc_units = nullptr;              // on-the-fly kernel: its CTAs' work (TcUnit)
     int64_t n_units = 0;
     int unit0_item = 0;                    // first item of the first unit (test hook)
@@ -59,6 +60,7 @@ struct DevicePlan {
     int64_t* tc_part_idx = nullptr;
     // symmetric CUDA-core translations (n_sym = 0: none), in batches (SymPlan)
     SymItem* sym_items = nullptr;
+    void* sym_block = nullptr;             // the allocation of the arrays below
     int64_t n_sym = 0, sym_slots = 0;      // items; slots of the largest batch
     SymRun* sym_runs = nullptr;
     int32_t* sym_idx = nullptr;

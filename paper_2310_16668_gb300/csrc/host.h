@@ -5,6 +5,7 @@
 
 #include <complex>
 #include <cstdint>
+#include <future>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -176,6 +177,7 @@ struct TcItem {                         // 64 bytes
 static_assert(sizeof(TcItem) == 64, "TcItem layout");
 
 struct Layout {
+    int threads = 0;                    // host threads of its builders (0 = all, 1 = the caller's only)
     int top = 1;
     int64_t n_tot = 0;
     std::vector<int64_t> box_off;       // nb, -1 if the box holds no entries
@@ -239,6 +241,11 @@ struct SymPlan {
     int64_t slots = 0;                  // of the largest batch
 };
 SymPlan make_sym_plan(const Layout& lay, int64_t max_slots);
+
+// how to run a part of a plan's preparation beside the rest: on a thread of its
+// own, or, for a small plan, with one thread or inside a parallel loop over
+// sets, when it is asked for
+std::launch host_task(const Layout& lay);
 
 // class of a tensor-core item's tile-list length (lengths within a factor
 // 1.25 share a class); items run longest class first

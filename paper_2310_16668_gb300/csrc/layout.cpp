@@ -23,7 +23,12 @@
 // arbitrarily close (or coincident) pairs.
 #include <algorithm>
 #include <cmath>
+#include <future>
 #include <numeric>
+
+#ifdef _OPENMP
+#include <omp.h>
+#endif
 
 #include "host.h"
 
@@ -31,7 +36,77 @@ namespace skel {
 
 namespace {
 constexpr int64_t kItemCost = 2048;   // source entries per warp work item
+constexpr int64_t kTaskEntries = 16384;   // from which a part of the preparation pays for a thread (50 us to start)
+// ---- symmetric CUDA-core translations ------------------------------------------
+// every task has its reverse (the neighbor relations are symmetric and so are
+// the masks), so each unordered pair of boxes is listed once, from its lower
+// box, and evaluated for both sides. Reads the boxes, tasks and chunks of lay.
+void list_sym_items(Layout& lay) {
+    const int64_t nb = (int64_t)lay.box_off.size();
+    auto slot_size = [&](int64_t b, int s) {
+        const int32_t* ss = &lay.slot_start[b * (kMaxSlots + 1)];
+        return (int64_t)(ss[s + 1] - ss[s]);
+    };
+    lay.entry_slot.assign(lay.n_tot, 0);
+    std::vector<uint8_t> chunk_slots(lay.chunk_start.size(), 0);
+    for (int64_t b = 0; b < nb; ++b) {
+        if (lay.box_off[b] < 0) continue;
+        const int32_t* ss = &lay.slot_start[b * (kMaxSlots + 1)];
+        for (int j = 0; j < lay.box_nslot[b]; ++j)
+            for (int32_t e = ss[j]; e < ss[j + 1]; ++e) {
+                lay.entry_slot[lay.box_off[b] + e] = (uint8_t)j;
+                chunk_slots[lay.box_chunk0[b] + e / kTcK] |= (uint8_t)(1 << j);
+            }
+    }
+    lay.sym_items.clear();
+    lay.sym_slots = 0;
+    int64_t up_pairs = 0, down_pairs = 0;                   // kept pairs of tasks to higher / lower boxes
+    for (int64_t b = 0; b < nb; ++b) {
+        if (lay.box_off[b] < 0) continue;
+        const int64_t tc0 = lay.box_chunk0[b], ntc = (lay.box_n[b] + kTcK - 1) / kTcK;
+        for (int64_t tk = lay.task_ptr[b]; tk < lay.task_ptr[b + 1]; ++tk) {
+            const int64_t src = lay.task_src[tk];
+            const uint64_t mask = lay.task_mask[tk];
+            int64_t kept = 0;
+            for (int i = 0; i < lay.box_nslot[b]; ++i)
+                for (int j = 0; j < lay.box_nslot[src]; ++j)
+                    if (!((mask >> (i * 8 + j)) & 1)) kept += slot_size(b, i) * slot_size(src, j);
+            if (src > b) up_pairs += kept;
+            if (src < b) down_pairs += kept;
+            if (src < b) continue;
+            const int64_t sc0 = lay.box_chunk0[src], nsc = (lay.box_n[src] + kTcK - 1) / kTcK;
+            const int per = sym_chunks(std::max(ntc, nsc));
+            for (int64_t i = 0; i < ntc; ++i) {
+                unsigned keeps = 0;                          // source slots that some slot of the target chunk keeps
+                for (int c = 0; c < kMaxSlots; ++c)
+                    if ((chunk_slots[tc0 + i] >> c) & 1) keeps |= ~(unsigned)(mask >> (8 * c)) & 0xFFu;
+                SymItem it{};
+                it.nsrc = 0;
+                for (int64_t j = src == b ? i : 0; j <= nsc; ++j) {
+                    const bool any = j < nsc && (chunk_slots[sc0 + j] & keeps);
+                    if (it.nsrc > 0 && (!any || it.nsrc == per)) {
+                        lay.sym_slots += 1 + it.nsrc;
+                        lay.sym_items.push_back(it);
+                        it.nsrc = 0;
+                    }
+                    if (!any) continue;
+                    if (it.nsrc == 0) {
+                        it.mask = mask;
+                        it.tchunk = (int32_t)(tc0 + i);
+                        it.schunk = (int32_t)(sc0 + j);
+                        it.flags = lay.task_flags[tk] | (src == b ? kSymSelf : 0);
+                    }
+                    ++it.nsrc;
+                }
+            }
+        }
+    }
+    if (up_pairs != down_pairs) {
+        lay.sym_items.clear();
+        lay.sym_slots = 0;
+    }
 }
+}  // namespace
 
 // class of a tile-list length: lengths within a factor 1.25 share a class
 int length_class(int n) {
@@ -275,6 +350,9 @@ void build_layout(const Plan& p, Layout& lay) {
             for (int d = 0; d < 4; ++d) lay.chunk_center.push_back(d < dim ? box_center(b, d) : 0.f);
         }
     }
+    // the symmetric translations are listed beside the tensor-core items, which
+    // take longer
+    std::future<void> sym = std::async(host_task(lay), [&lay] { list_sym_items(lay); });
     // one item: rows [row_off, row_off + nrows) whose slot j covers rows
     // [sst[j], sst[j+1]); targets = (box, first slot of that box in the item,
     // row of the box's first entry)
@@ -379,73 +457,16 @@ void build_layout(const Plan& p, Layout& lay) {
     lay.tc_n_slots = slot;
     to_csr(parts, lay.tc_part_ptr, lay.tc_part_idx);
 
-    // ---- symmetric CUDA-core translations ------------------------------------------
-    // every task has its reverse (the neighbor relations are symmetric and so
-    // are the masks), so each unordered pair of boxes is listed once, from its
-    // lower box, and evaluated for both sides
-    lay.entry_slot.assign(lay.n_tot, 0);
-    for (int64_t b = 0; b < nb; ++b) {
-        if (lay.box_off[b] < 0) continue;
-        const int32_t* ss = &lay.slot_start[b * (kMaxSlots + 1)];
-        for (int j = 0; j < lay.box_nslot[b]; ++j)
-            for (int32_t e = ss[j]; e < ss[j + 1]; ++e) lay.entry_slot[lay.box_off[b] + e] = (uint8_t)j;
-    }
-    lay.sym_items.clear();
-    lay.sym_slots = 0;
-    auto slots_of = [&](int64_t chunk) {
-        unsigned m = 0;
-        for (int32_t e = 0; e < lay.chunk_cnt[chunk]; ++e) m |= 1u << lay.entry_slot[lay.chunk_start[chunk] + e];
-        return m;
-    };
-    std::vector<uint8_t> chunk_slots(lay.chunk_start.size());
-    for (size_t c = 0; c < chunk_slots.size(); ++c) chunk_slots[c] = (uint8_t)slots_of((int64_t)c);
-    int64_t up_pairs = 0, down_pairs = 0;                   // kept pairs of tasks to higher / lower boxes
-    for (int64_t b = 0; b < nb; ++b) {
-        if (lay.box_off[b] < 0) continue;
-        const int64_t tc0 = lay.box_chunk0[b], ntc = (lay.box_n[b] + kTcK - 1) / kTcK;
-        for (int64_t tk = lay.task_ptr[b]; tk < lay.task_ptr[b + 1]; ++tk) {
-            const int64_t src = lay.task_src[tk];
-            const uint64_t mask = lay.task_mask[tk];
-            int64_t kept = 0;
-            for (int i = 0; i < lay.box_nslot[b]; ++i)
-                for (int j = 0; j < lay.box_nslot[src]; ++j)
-                    if (!((mask >> (i * 8 + j)) & 1)) kept += slot_size(b, i) * slot_size(src, j);
-            if (src > b) up_pairs += kept;
-            if (src < b) down_pairs += kept;
-            if (src < b) continue;
-            const int64_t sc0 = lay.box_chunk0[src], nsc = (lay.box_n[src] + kTcK - 1) / kTcK;
-            const int per = sym_chunks(std::max(ntc, nsc));
-            for (int64_t i = 0; i < ntc; ++i) {
-                SymItem it{};
-                it.nsrc = 0;
-                for (int64_t j = src == b ? i : 0; j <= nsc; ++j) {
-                    bool any = false;                        // some pair of slots of the two chunks is kept
-                    if (j < nsc)
-                        for (int c = 0; c < kMaxSlots; ++c)
-                            if (((chunk_slots[tc0 + i] >> c) & 1) &&
-                                (chunk_slots[sc0 + j] & ~(unsigned)(mask >> (8 * c)) & 0xFFu))
-                                any = true;
-                    if (it.nsrc > 0 && (!any || it.nsrc == per)) {
-                        lay.sym_slots += 1 + it.nsrc;
-                        lay.sym_items.push_back(it);
-                        it.nsrc = 0;
-                    }
-                    if (!any) continue;
-                    if (it.nsrc == 0) {
-                        it.mask = mask;
-                        it.tchunk = (int32_t)(tc0 + i);
-                        it.schunk = (int32_t)(sc0 + j);
-                        it.flags = lay.task_flags[tk] | (src == b ? kSymSelf : 0);
-                    }
-                    ++it.nsrc;
-                }
-            }
-        }
-    }
-    if (up_pairs != down_pairs) {
-        lay.sym_items.clear();
-        lay.sym_slots = 0;
-    }
+    sym.get();
+}
+
+std::launch host_task(const Layout& lay) {
+    bool here = lay.threads == 1 || lay.n_tot < kTaskEntries;
+#ifdef _OPENMP
+    here |= omp_in_parallel() != 0;
+#endif
+    // (with both flags a thread that cannot be started is run by get())
+    return here ? std::launch::deferred : std::launch::async | std::launch::deferred;
 }
 
 SymPlan make_sym_plan(const Layout& lay, int64_t max_slots) {

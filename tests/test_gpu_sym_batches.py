@@ -51,3 +51,12 @@ def test_slots_take_bounded_memory():
     one, two = (SkelFMM(x, "laplace3d", 1e-6, 128, nrhs_max=m, device_build=True).info() for m in (1, 2))
     grown = two["device_bytes"] - one["device_bytes"]
     assert grown <= 2 * 12 * one["n_index"] + 32 * 12 * one["n_work_items"] + BATCH * 32 * 8, grown
+
+
+@pytest.mark.parametrize("kind,n", [("laplace3d", 40000), ("laplace2d", 30000)])
+def test_host_threads_change_no_bit(kind, n):
+    """The items, batches and slots are listed by many host threads or one."""
+    x = clustered(n, 3 if kind.endswith("3d") else 2, 98)
+    q = torch.from_numpy(W.charges_normal(x.shape[0], 2, 99)).cuda()
+    one, many = (SkelFMM(x, kind, 1e-6, 64, nrhs_max=2, num_threads=t).apply(q, "fp64") for t in (1, 0))
+    assert torch.equal(one, many)

@@ -427,6 +427,16 @@ int skel_test_fail_alloc(int countdown);
 int skel_test_set_updown(skel_handle h, int code);
 
 /*
+ * skel_test_units — how the on-the-fly tensor-core translations of h (real
+ * kernels) are divided, for tests that mean to reach a form: out5 = CTAs with
+ * one item, with two items that share their tiles, with two unrelated items;
+ * items whose tile lists are cut over several CTAs; tiles of the longest
+ * piece. All 0 for complex kernels.
+ * Errors: SKEL_ERR_ARG (NULL), SKEL_ERR_STATE (host-only plan).
+ */
+int skel_test_units(skel_handle h, int64_t* out5);
+
+/*
  * skel_autotune — pick, by measurement on this plan and device, the variants
  * the FP32 applies of nrhs right-hand sides will use: per tree level and
  * direction the launch shape of the up/down kernel (1, 2, 4 or 8 warps per

@@ -437,7 +437,7 @@ void permute(bool out, const DevicePlan* dp, const S* src, S* dst, int nrhs, cud
 }
 
 constexpr int64_t kResidentGroups = 4 * 152;   // groups of the on-the-fly kernel that run at a time
-constexpr int32_t kWholeList = INT32_MAX / 2 / kTcGroup * kTcGroup;
+constexpr int32_t kWholeList = 1 << 30;
 
 constexpr int kProfEvents = 8;   // 7 phase boundaries + the start of the main translation kernel
 constexpr int kMainEvent = 7;
@@ -856,7 +856,7 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
 // against 233, 65,536 (116) 777 against 965 (share: a quarter of the tiles per
 // resident group); 2D N = 65,536 454 against 303 (before tc_log8). There, and for pairs in plans
 // with a little more work, long lists are cut into parts of whole segments
-// (kTcGroup tiles); tc_segments_kernel adds the segments of a cut item.
+// (TcItem::lseg); tc_segments_kernel adds the segments of a cut item.
 // Neither pairing nor cutting changes a result.
 constexpr int64_t kPairShare = 16;             // share from which 3D items share CTAs
 constexpr int64_t kCutShare = 256;             // ... up to which long lists are cut
@@ -872,7 +872,10 @@ Units make_units(const std::vector<TcItem>& items, int dim) {
     for (size_t i = 0; i < items.size(); ++i) tiles += len((int32_t)i);
     // a part: about a quarter of what each resident group gets in all
     const int64_t share = tiles / (4 * kResidentGroups);
-    const int cut = (int)std::max<int64_t>(1, (share + kTcGroup / 2) / kTcGroup) * kTcGroup;
+    auto cut = [&](int32_t i) {
+        const int64_t seg = (int64_t)1 << items[i].lseg;
+        return (int)(std::max<int64_t>(1, (share + seg / 2) / seg) * seg);
+    };
     const bool small = share < kCutShare, pairs = dim == 3 && share >= kPairShare;
     Units r;
     r.part0.assign(items.size(), -1);
@@ -899,21 +902,21 @@ Units make_units(const std::vector<TcItem>& items, int dim) {
     for (size_t i = 0; i < items.size(); ++i) {
         if (mate[i] == -2) continue;
         const int n = len((int32_t)i);
-        const bool split = small && n > cut;
-        const int step = split ? cut : std::max(n, 1);
+        const bool split = small && n > cut((int32_t)i);
+        const int step = split ? cut((int32_t)i) : std::max(n, 1);
         for (int t = 0; t < std::max(n, 1); t += step)
             pieces.push_back(Piece{(int32_t)i, mate[i], t, std::min(step, n - t)});
         if (!split) continue;
         for (int32_t it : {(int32_t)i, mate[i]}) {
             if (it < 0) continue;
             r.part0[it] = r.segments;
-            r.segments += (n + kTcGroup - 1) / kTcGroup;
+            r.segments += (n + (1 << items[it].lseg) - 1) >> items[it].lseg;
             r.split.push_back(it);
         }
     }
     std::stable_sort(pieces.begin(), pieces.end(),
                      [](const Piece& x, const Piece& y) { return length_class(x.n) > length_class(y.n); });
-    auto count = [&](const Piece& p) { return r.part0[p.a] >= 0 ? cut : kWholeList; };
+    auto count = [&](const Piece& p) { return r.part0[p.a] >= 0 ? cut(p.a) : kWholeList; };
     const Piece* single = nullptr;
     for (const Piece& p : pieces) {
         if (p.b >= 0) {
@@ -1255,6 +1258,15 @@ DevicePlan* device_plan_create(const Plan& p, const Layout& lay, int nrhs_max, i
             dp->unit_block = upload_all<TcUnit, int64_t, int32_t>(dp->bytes, {u.units, &units}, {u.part0, &part0},
                                                                   {u.split, &dp->tc_split});
             dp->tc_units = units;
+            for (const TcUnit& x : u.units) {
+                UnitStats& s = dp->unit_stats;
+                (x.b < 0 ? s.single : x.shared ? s.shared : s.unrelated) += 1;
+                for (int g = 0; g < (x.b < 0 ? 1 : 2); ++g) {
+                    const TcItem& it = lay.tc_items[g ? x.b : x.a];
+                    s.longest = std::max<int64_t>(s.longest, std::min(x.count, it.list_hi - it.list_lo - (g ? x.lo_b : x.lo_a)));
+                }
+            }
+            dp->unit_stats.cut = dp->n_split;
             if (dp->n_split > 0) {
                 dp->tc_part0 = part0;
                 dp->tc_parts = dalloc<float>((size_t)u.segments * kTcRows * kTcN, dp->bytes);

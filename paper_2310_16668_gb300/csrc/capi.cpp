@@ -797,6 +797,16 @@ int skel_test_set_updown(skel_handle h, int code) {
     });
 }
 
+int skel_test_units(skel_handle h, int64_t* out5) {
+    return guarded([&] {
+        if (!h || !out5) throw Error(SKEL_ERR_ARG, "NULL argument");
+        if (!h->dev) throw Error(SKEL_ERR_STATE, "plan was built host-only");
+        const skel::UnitStats& s = h->dev->unit_stats;
+        const int64_t v[5] = {s.single, s.shared, s.unrelated, s.cut, s.longest};
+        std::copy(v, v + 5, out5);
+    });
+}
+
 int skel_autotune(skel_handle h, int nrhs, int allow_store, void* stream, skel_tuning* out) {
     return guarded([&] {
         if (!h) throw Error(SKEL_ERR_ARG, "handle is NULL");

@@ -11,6 +11,12 @@ namespace skel {
 
 struct DeviceBuffers;   // per precision (defined in apply.cu)
 
+// CTAs of the on-the-fly kernel by form, items whose lists are cut, and the
+// longest piece of a list in tiles
+struct UnitStats {
+    int64_t single = 0, shared = 0, unrelated = 0, cut = 0, longest = 0;
+};
+
 struct DevicePlan {
     int device = 0;
     int dim = 3, kind = 1;
@@ -55,6 +61,7 @@ struct DevicePlan {
     float* tc_parts = nullptr;
     int32_t* tc_split = nullptr;           // the cut items
     int64_t n_split = 0;
+    UnitStats unit_stats;                  // (test hook)
     int64_t tc_n_slots = 0;
     int64_t* tc_part_ptr = nullptr;        // per entry: its partial sums (tensor-core mode)
     int64_t* tc_part_idx = nullptr;

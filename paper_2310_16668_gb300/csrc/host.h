@@ -169,12 +169,25 @@ static_assert(sizeof(SrcTile) == 64, "SrcTile is one 64-byte bulk copy");
 struct TcItem {                         // 64 bytes
     int64_t row_off;                    // entry of row 0
     int32_t nrows;                      // valid rows (<= 128)
-    int32_t nslot;
+    int16_t nslot;
+    int16_t lseg;                       // its tiles are summed in segments of 2^lseg (see tc_segment)
     int32_t slot_start[kMaxSlots + 1];  // first row of each slot (may be < 0 for a box's later rows)
     int32_t list_lo, list_hi;           // its tiles: [list_lo, list_hi) of tc_tiles
     int32_t box;                        // the box whose rows these are (-1: packed leaves)
 };
 static_assert(sizeof(TcItem) == 64, "TcItem layout");
+
+// log2 of the tiles of a segment, the shortest piece into which the on-the-fly
+// kernel can cut an item's list: 128 tiles, and 16 where a 3D plan has so few
+// that its lists (about 60 tiles) would each be one piece and leave most of the
+// chip idle. Near kernel, 32 right-hand sides, leaves of 128, segments of 128, 32
+// and 16 (and one item per CTA, two threads per row, before): N = 1,500 46, 43, 29
+// (42) us, 3,000 79, 43, 38 (69), 5,000 119, 56, 60 (103), 7,000 (12,187 tiles)
+// 124, 90, 82. From N = 8,000 (18,077 tiles) segments of 128 are faster than that
+// kernel (131, 137) and leave larger plans fewer sums to add up. Fixed with the item, so that a
+// merged plan gives each set its own plan's sums.
+constexpr int64_t kShortTiles = 14592;  // 24 for each of the 608 groups of rows that run at a time
+constexpr int tc_segment(int dim, int64_t tiles) { return dim == 3 && tiles < kShortTiles ? 4 : 7; }
 
 struct Layout {
     int threads = 0;                    // host threads of its builders (0 = all, 1 = the caller's only)

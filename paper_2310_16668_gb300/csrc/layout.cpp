@@ -382,7 +382,7 @@ void build_layout(const Plan& p, Layout& lay) {
         TcItem it{};
         it.row_off = row_off;
         it.nrows = nrows;
-        it.nslot = nslot;
+        it.nslot = (int16_t)nslot;
         for (int j = 0; j <= nslot; ++j) it.slot_start[j] = sst[j];
         it.list_lo = (int32_t)lay.tc_tiles.size();
         for (size_t k = 0; k < srcs.size(); ++k) {
@@ -445,6 +445,7 @@ void build_layout(const Plan& p, Layout& lay) {
         sst[tg.size()] = rows;
         emit(row_off, rows, (int)tg.size(), sst, tg);
     }
+    for (TcItem& it : lay.tc_items) it.lseg = (int16_t)tc_segment(dim, (int64_t)lay.tc_tiles.size());
     // longest lists first, so that the long items start early, by classes of
     // lengths within 25% of each other; within a class the items keep their
     // order (boxes in level and Morton order), so that items running at the

@@ -37,7 +37,6 @@ constexpr int kTcCompute = 128 * kTpr;         // compute threads
 constexpr int kSrcPerThread = 32 / kTpr;       // sources of a tile each compute thread evaluates
 constexpr int kTcThreads = kTcCompute + 64;    // + the producer warp and the MMA warp
 constexpr int kTcN = 32;                       // right-hand sides per pass (MMA N)
-constexpr int kTcGroup = 128;                  // tiles of a segment (summed in registers; segments add up in U)
 constexpr int kTcOuter = 128;                  // symmetric store, complex kernel: tiles summed in registers
                                                // before the outer sum
 constexpr int kNA = 3;                         // A-operand buffers in tensor memory
@@ -93,8 +92,8 @@ static_assert(sizeof(ItemSym) == 40, "ItemSym layout");
 struct TcUnit {
     int32_t a, b;                              // items; b = -1: one item
     int32_t shared;
-    int32_t lo_a, lo_b;                        // first tile of each item's list (a multiple of kTcGroup)
-    int32_t count;                             // tiles from there, at most (a multiple of kTcGroup)
+    int32_t lo_a, lo_b;                        // first tile of each item's list (where a segment starts)
+    int32_t count;                             // tiles from there, at most (whole segments)
 };
 
 struct TcArgs {
@@ -448,11 +447,12 @@ constexpr int kNAS = 2;                        // A buffers
 constexpr uint32_t kColSL = 64, kColSA = 128;
 
 // The stored kernels' MMAs of tile m (its B operand at bh): the sum of
-// tc_near.cuh, with pair p's hi*hi products in D[p % 2]
-__device__ __forceinline__ void tcs_mma_tile(uint32_t tbase, int m, uint32_t bh, uint32_t idesc) {
+// tc_near.cuh, with pair p's hi*hi products in D[p % 2]; mask: tiles of a
+// segment - 1
+__device__ __forceinline__ void tcs_mma_tile(uint32_t tbase, int m, int mask, uint32_t bh, uint32_t idesc) {
     const uint32_t d = tbase + kColD + 32u * ((uint32_t)(m >> 1) & 1u), l = tbase + kColSL;
     const uint32_t ahi = tbase + kColSA + 64u * (uint32_t)(m % kNAS), alo = ahi + 32u, b0 = smem_desc_lo(bh);
-    const bool first = !(m & 1), seg = (m & (kTcGroup - 1)) == 0;
+    const bool first = !(m & 1), seg = (m & mask) == 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const uint32_t dbh = b0 + kDescStep * k, dbl = dbh + kDescLoPart;
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
     const TcItem* itp = a.items + blockIdx.x;
     const int64_t row_off = itp->row_off;
     const int nrows = itp->nrows, list_lo = itp->list_lo;
-    const int ntile = itp->list_hi - list_lo;
+    const int ntile = itp->list_hi - list_lo, mask = (1 << itp->lseg) - 1;
 
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
                 const int s = m % NST;
                 if (!mbar_wait(sm_addr(&S.afull[s]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tcs_mma_tile(tbase, m, sm_addr(S.st[s].b), idesc);
+                tcs_mma_tile(tbase, m, mask, sm_addr(S.st[s].b), idesc);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.empty[s])) : "memory");
             }
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
         // the segment that ends before tile u goes to U
         auto flush = [&](int u) {
             if (u > 0) done(u - 1);
-            const int s0 = u > 0 ? (u - 1) & ~(kTcGroup - 1) : 0;
+            const int s0 = u > 0 ? (u - 1) & ~mask : 0;
             float v[kCols];
             sums.finish(tcol, u - s0, v);
             if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
@@ -637,12 +637,12 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
                     glo[jj + 1] = __float_as_uint(lo.y);
                 }
             }
-            if (u > 0 && (u & (kTcGroup - 1)) == 0) {
+            if (u > 0 && (u & mask) == 0) {
                 flush(u);
             } else {
                 if (u >= 2) done(u - 2);
                 // before the pair that starts with tile u, the pair two before it
-                if (!(u & 1) && (u & (kTcGroup - 1)) >= 4) sums.pair(tcol, ((u & (kTcGroup - 1)) >> 1) - 2);
+                if (!(u & 1) && (u & mask) >= 4) sums.pair(tcol, ((u & mask) >> 1) - 2);
             }
             const uint32_t acol = tbase + lane_off + kColSA + 64u * (u % kNAS) + (uint32_t)j0;
             tmem_st16(acol, ghi);

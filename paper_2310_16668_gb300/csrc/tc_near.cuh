@@ -24,7 +24,7 @@
 // 66 -> 43.
 //
 // The sum, the same for all forms and for the stored kernels (so all give
-// the same bits): an item's tile list is cut into segments of kTcGroup tiles
+// the same bits): an item's tile list is cut into segments of 128 tiles (16 in small 3D plans, tc_segment)
 // and a segment into pairs of tiles. The hi*hi products of a pair accumulate in
 // tensor memory (D: 8 K-steps) and are then added to an FP32 register sum;
 // the hi*lo and lo*hi products of the whole segment accumulate in a second
@@ -284,7 +284,7 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
     constexpr int NC = SPLIT ? 16 : 32;                    // accumulator columns of a thread
     const int warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
     const TcItem* itp = a.items + item;
-    const int nrows = itp->nrows, list_lo = itp->list_lo;
+    const int nrows = itp->nrows, list_lo = itp->list_lo, lseg = itp->lseg;
     // warp w always runs on scheduler w % 4: the 32-row blocks are dealt to the
     // warps from a position that moves with the CTA
     const int blk = (warp + rot) & 3, row = 32 * blk + lane;
@@ -345,7 +345,7 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
     uint32_t ph = 0u;
     int s0 = t_lo;
     do {                                                   // segments (an item without tiles writes zeros)
-        const int send = min(s0 + kTcGroup, t_hi);
+        const int send = min(s0 + (1 << lseg), t_hi);
 #pragma unroll
         for (int c = 0; c < NC / 2; ++c) acc[c] = make_float2(0.f, 0.f);
         tmem_zero<NC>(dcol);
@@ -472,12 +472,12 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
                 tc_add_rows<KIND, NC>(a, urow, c0, s0 > 0, v);
             } else {
                 // a part of the item: its segments go to their own rows
-                float4* d = reinterpret_cast<float4*>(parts + ((int64_t)(s0 / kTcGroup) * kTcRows + row) * kTcN + c0);
+                float4* d = reinterpret_cast<float4*>(parts + ((int64_t)(s0 >> lseg) * kTcRows + row) * kTcN + c0);
 #pragma unroll
                 for (int c = 0; c < NC / 4; ++c) d[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
             }
         }
-        s0 += kTcGroup;
+        s0 += 1 << lseg;
     } while (s0 < t_hi);
     return ok;
 }
@@ -666,7 +666,7 @@ template <int KIND>
 __global__ void __launch_bounds__(256) tc_segments_kernel(const TcArgs a, const int32_t* __restrict__ split) {
     const int item = split[blockIdx.x];
     const TcItem it = a.items[item];
-    const int nseg = (it.list_hi - it.list_lo + kTcGroup - 1) / kTcGroup;
+    const int nseg = (it.list_hi - it.list_lo + (1 << it.lseg) - 1) >> it.lseg;
     const float scale = (float)green_scale<KIND>();
     const float* parts = a.parts + a.part0[item] * (kTcRows * kTcN);
     for (int i = threadIdx.x; i < it.nrows * (kTcN / 4); i += 256) {

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
     const TcItem* itp = a.items + blockIdx.x;
     const int64_t row_off = itp->row_off;
     const int nrows = itp->nrows, list_lo = itp->list_lo;
-    const int ntile = itp->list_hi - list_lo;
+    const int ntile = itp->list_hi - list_lo, mask = (1 << itp->lseg) - 1;
 
     if (tid == 0) {
         for (int s = 0; s < NA; ++s) {
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
                 if (!mbar_wait(sm_addr(&S.afull[sa]), (uint32_t)((m / NA) & 1), a.wait_ns)) err = true;
                 if (!mbar_wait(sm_addr(&S.fullB[sb]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                tcs_mma_tile(tbase, m, sm_addr(S.bb[sb].b), idesc);
+                tcs_mma_tile(tbase, m, mask, sm_addr(S.bb[sb].b), idesc);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                              :: "r"(sm_addr(&S.emptyB[sb])) : "memory");
             }
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
         // the segment that ends before tile u goes to U
         auto flush = [&](int u) {
             if (u > 0) done(u - 1);
-            const int s0 = u > 0 ? (u - 1) & ~(kTcGroup - 1) : 0;
+            const int s0 = u > 0 ? (u - 1) & ~mask : 0;
             float v[kCols];
             sums.finish(tcol, u - s0, v);
             if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
@@ -181,12 +181,12 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
                     glo[jj + 1] = __float_as_uint(lo.y);
                 }
             }
-            if (u > 0 && (u & (kTcGroup - 1)) == 0) {
+            if (u > 0 && (u & mask) == 0) {
                 flush(u);
             } else {
                 if (u >= 2) done(u - 2);
                 // before the pair that starts with tile u, the pair two before it
-                if (!(u & 1) && (u & (kTcGroup - 1)) >= 4) sums.pair(tcol, ((u & (kTcGroup - 1)) >> 1) - 2);
+                if (!(u & 1) && (u & mask) >= 4) sums.pair(tcol, ((u & mask) >> 1) - 2);
             }
             const uint32_t acol = tbase + lane_off + kColSA + 64u * (u % kNAS) + (uint32_t)j0;
             tmem_st16(acol, ghi);

@@ -76,3 +76,28 @@ def test_merged_plans_keep_their_sets_segments():
         one = torch.empty((nrhs, len(sets[i])), device="cuda")
         f.apply_into(q[:, at].contiguous(), one, nrhs, "fp32_tc")
         assert torch.equal(one, u[:, at]), i
+
+
+@pytest.mark.parametrize("kind,n,leaf,form", [
+    ("laplace3d", 30000, 128, "pairs, cut"),
+    ("laplace3d", 16500, 16500, "pairs, cut"),           # one leaf: 129 items, the last one of 116 rows
+    ("laplace3d", 120000, 128, "pieces of two segments"),
+    ("laplace3d", 150000, 128, "pairs, whole lists"),    # the form of every larger 3D plan
+    ("laplace2d", 4300, 4300, "single, cut"),
+])
+@pytest.mark.parametrize("nrhs", [4, 33])
+def test_forms_match_fp64(kind, n, leaf, form, nrhs):
+    x = W.points_uniform(n, int(kind[-2]), 75)
+    f = SkelFMM(x, kind, 1e-6, leaf, nrhs_max=nrhs, device_build=n > 60000)
+    un = _units(f)
+    if form.startswith("single"):
+        assert un["single"] > 0 and un["cut"] > 0 and un["shared"] == un["unrelated"] == 0
+    else:
+        assert un["shared"] > 0 and un["unrelated"] > 0
+        if form == "pairs, cut":
+            assert un["cut"] > 0 and un["longest"] == 128
+        elif form == "pieces of two segments":
+            assert un["cut"] > 0 and un["longest"] == 256
+        else:
+            assert un["cut"] == 0 and un["longest"] > 256
+    _check(f, n, nrhs, 76)

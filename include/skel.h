@@ -418,9 +418,10 @@ int skel_test_fail_alloc(int countdown);
  * upward and downward pass on h (what skel_autotune otherwise picks per
  * level): code 0 = the default rule, 1 / 2 / 4 / 8 = the plain kernel with
  * that many warps per CTA, 17 / 18 / 20 / 24 = the asynchronous-copy kernel
- * with 1 / 2 / 4 / 8 warps. Every shape gives the same result bit for bit,
- * which tests check with it. Applies of up to 8 right-hand sides have one
- * shape of their own, whatever the code.
+ * with 1 / 2 / 4 / 8 warps, 33 / 40 = the kernel with a row per lane with 1 / 8
+ * warps per 32 rows (up to 8 right-hand sides; the default rule for wider
+ * applies). Every shape gives the same result bit for bit, which tests check
+ * with it.
  * Errors: SKEL_ERR_ARG (NULL handle, other codes), SKEL_ERR_STATE (host-only
  * plan).
  */
@@ -442,8 +443,9 @@ int skel_test_units(skel_handle h, int64_t* out5);
  * direction the launch shape of the up/down kernel (1, 2, 4 or 8 warps per
  * CTA sharing a 32-row block, with the blocks staged through registers or by
  * asynchronous copies; every shape adds the same partial sums in the same
- * order; up to 8 right-hand sides have one shape, which leaves nothing to
- * choose: the settings of wider applies then stay as they are), and for the tensor-core
+ * order; up to 8 right-hand sides have two more shapes, a row per lane, and
+ * settings of their own, so that tuning for few and for many right-hand sides
+ * do not disturb each other), and for the tensor-core
  * translations (real kernels, nrhs >= 4) whether the
  * kernel values are evaluated on the fly or read from a store (the choice
  * between operators stored and evaluated on the fly: the per-tile and the
@@ -464,8 +466,7 @@ typedef struct {
     double ms_stored;         /* the same reading the per-tile store (-1: not timed)            */
     int    stored;            /* store mode the plan keeps after tuning: 0 none, 1 per-tile,
                                  2 symmetric                                                     */
-    int    n_updown;          /* up/down level launches tuned (levels x 2 directions; 0 for up
-                                 to 8 right-hand sides)                                         */
+    int    n_updown;          /* up/down level launches tuned (levels x 2 directions)           */
     int    n_changed;         /* of those, choices unlike the default rule                      */
     double ms_updown_default; /* their summed time with the default rule                        */
     double ms_updown_tuned;   /* and with the chosen variants                                   */

@@ -331,14 +331,13 @@ int up_down_tc(bool down, DevicePlan* dp, int l, float* X, int nrhs, cudaStream_
 }
 
 template <class S, bool DOWN, int RT>
-void ud_narrow_launch_rt(const DevicePlan* dp, int l, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
+void ud_few_launch_rt(const DevicePlan* dp, int l, int W, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
     const std::vector<int64_t>& ptr = dp->ud_work_ptr[DOWN ? 1 : 0][0];
     const int64_t w0 = ptr[l], n = ptr[l + 1] - w0;
     if (n <= 0) return;
     const int2* work = dp->ud_work[DOWN ? 1 : 0][0] + w0;
     constexpr int th = 32 * kUnWarps;
-    const int ninner = DOWN ? dp->up_level_maxk[l] : dp->up_level_maxr[l];
-    if (ninner <= 2 * un_segment(0))
+    if (W == 1)
         updown_narrow_kernel<S, DOWN, RT, 1><<<ceil_div(n, kUnWarps), th, 0, st>>>(dp->up, work, (int)n, dp->pos, T, X,
                                                                                   nrhs, conj_op);
     else
@@ -346,41 +345,53 @@ void ud_narrow_launch_rt(const DevicePlan* dp, int l, int nrhs, const S* T, S* X
                                                                                 nrhs, conj_op);
 }
 template <class S, bool DOWN>
-void ud_narrow_launch(const DevicePlan* dp, int l, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
-    if (nrhs == 1) ud_narrow_launch_rt<S, DOWN, 1>(dp, l, nrhs, T, X, conj_op, st);
-    else if (nrhs == 2) ud_narrow_launch_rt<S, DOWN, 2>(dp, l, nrhs, T, X, conj_op, st);
-    else if (nrhs <= 4) ud_narrow_launch_rt<S, DOWN, 4>(dp, l, nrhs, T, X, conj_op, st);
-    else if constexpr (sizeof(S) <= 8) ud_narrow_launch_rt<S, DOWN, 8>(dp, l, nrhs, T, X, conj_op, st);
+void ud_few_launch(const DevicePlan* dp, int l, int W, int nrhs, const S* T, S* X, bool conj_op, cudaStream_t st) {
+    if (nrhs == 1) ud_few_launch_rt<S, DOWN, 1>(dp, l, W, nrhs, T, X, conj_op, st);
+    else if (nrhs == 2) ud_few_launch_rt<S, DOWN, 2>(dp, l, W, nrhs, T, X, conj_op, st);
+    else if (nrhs <= 4) ud_few_launch_rt<S, DOWN, 4>(dp, l, W, nrhs, T, X, conj_op, st);
+    else if constexpr (sizeof(S) <= 8) ud_few_launch_rt<S, DOWN, 8>(dp, l, W, nrhs, T, X, conj_op, st);
 }
 
-// few right-hand sides: a row per lane instead of a column (every launch shape
-// of the other kernels puts 32 columns on the lanes)
+// few right-hand sides: updown_narrow_kernel (a row per lane instead of a
+// column) serves them too
+constexpr int kUdFew = 32;                 // launch-shape codes: kUdFew + its W
 template <class S>
-constexpr bool ud_narrow(int nrhs) {
+constexpr bool ud_few(int nrhs) {
     return nrhs <= (sizeof(S) <= 8 ? kUnMaxRhs : 4);
 }
+// the default: a warp per stream (W = 8), unless the level has as many work
+// entries as such CTAs run at a time and short sums. 4 right-hand sides, W = 8
+// against W = 1: 1,016 entries of up to 61 inner indices 10.4, 14.5 us; 1,024 of
+// 56 10.8, 8.3; 2,054 of 56 14.9, 12.4; 5,705 of 21 30.8, 14.9; 1,504 of 129 14.9,
+// 20.6; 384 of 797 14.5, 39.4
+inline int ud_few_default(int ninner, int64_t work) { return kUdFew + (ninner <= 128 && work >= 1024 ? 1 : kUnWarps); }
 
-// one level of the upward or downward pass; warps = 0: the level's setting
+// one level of the upward or downward pass; shape = 0: the level's setting
 // (autotuned for FP32, else the default rule)
 template <class S>
 void up_down(bool down, const DevicePlan* dp, int l, const S* T, S* X, int nrhs, bool conj_op, cudaStream_t st,
-             int warps = 0) {
-    if (ud_narrow<S>(nrhs)) {
-        down ? ud_narrow_launch<S, true>(dp, l, nrhs, T, X, conj_op, st)
-             : ud_narrow_launch<S, false>(dp, l, nrhs, T, X, conj_op, st);
-        return;
-    }
+             int shape = 0) {
     ud_attributes_once<S>();
     const int64_t b0 = dp->up_level_ptr[l], b1 = dp->up_level_ptr[l + 1];
     const int nout = down ? dp->up_level_maxr[l] : dp->up_level_maxk[l];
     const int ninner = down ? dp->up_level_maxk[l] : dp->up_level_maxr[l];
     const dim3 grid((unsigned)(b1 - b0), std::max(1u, ceil_div(nout, kGT)), ceil_div(nrhs, kGT));
-    int W = warps;
+    const bool few = ud_few<S>(nrhs);
+    int W = shape;
     if (W == 0 && std::is_same<S, float>::value) {
-        const std::vector<int8_t>& t = down ? dp->ud_warps_down : dp->ud_warps_up;
+        const std::vector<int8_t>& t = few ? (down ? dp->ud_few_down : dp->ud_few_up)
+                                           : (down ? dp->ud_warps_down : dp->ud_warps_up);
         if (l < (int)t.size() && t[l] > 0) W = t[l];
     }
-    if (W == 0) W = ud_default_warps((ninner + kGT - 1) / kGT);
+    if (W == 0) {
+        const std::vector<int64_t>& work = dp->ud_work_ptr[down ? 1 : 0][0];
+        W = few ? ud_few_default(ninner, work[l + 1] - work[l]) : ud_default_warps((ninner + kGT - 1) / kGT);
+    }
+    if (W > kUdFew) {
+        down ? ud_few_launch<S, true>(dp, l, W - kUdFew, nrhs, T, X, conj_op, st)
+             : ud_few_launch<S, false>(dp, l, W - kUdFew, nrhs, T, X, conj_op, st);
+        return;
+    }
     const UpBox* up = dp->up + b0;
     if constexpr (std::is_same<S, float>::value) {
         if (W > kUdAsync) {
@@ -1450,22 +1461,27 @@ TuneReport device_autotune(DevicePlan* dp, int nrhs, bool allow_store, void* str
         };
         // 1. up/down launch shape per level: warps per CTA (every choice
         //    adds the same partial sums in the same order); few right-hand
-        //    sides have one shape, and the settings of the others stay
-        const int nl = ud_narrow<float>(nrhs) ? 0 : (int)dp->up_level_ptr.size() - 1;
-        if (nl > 0) {
-            dp->ud_warps_up.assign(nl, 0);
-            dp->ud_warps_down.assign(nl, 0);
-        }
+        //    sides have two more shapes and settings of their own
+        const bool few = ud_few<float>(nrhs);
+        const int nl = (int)dp->up_level_ptr.size() - 1;
+        std::vector<int8_t>& t_up = few ? dp->ud_few_up : dp->ud_warps_up;
+        std::vector<int8_t>& t_down = few ? dp->ud_few_down : dp->ud_warps_down;
+        t_up.assign(std::max(nl, 0), 0);
+        t_down.assign(std::max(nl, 0), 0);
         for (int l = 2; l <= dp->L && l < nl; ++l) {
             if (dp->up_level_ptr[l + 1] == dp->up_level_ptr[l]) continue;
             for (int down = 0; down < 2; ++down) {
-                std::vector<int8_t>& t = down ? dp->ud_warps_down : dp->ud_warps_up;
+                std::vector<int8_t>& t = down ? t_down : t_up;
                 const float* T = (const float*)(down ? b->Tt : b->T);
                 const int ninner = down ? dp->up_level_maxk[l] : dp->up_level_maxr[l];
-                const int def = ud_default_warps((ninner + kGT - 1) / kGT);
+                const std::vector<int64_t>& work = dp->ud_work_ptr[down][0];
+                const int def = few ? ud_few_default(ninner, work[l + 1] - work[l])
+                                    : ud_default_warps((ninner + kGT - 1) / kGT);
                 double best_ms = 1e30, def_ms = 0;
                 int best = def;
-                for (int W : {1, 2, 4, 8, kUdAsync + 1, kUdAsync + 2, kUdAsync + 4, kUdAsync + 8}) {
+                for (int W : {1, 2, 4, 8, kUdAsync + 1, kUdAsync + 2, kUdAsync + 4, kUdAsync + 8, kUdFew + 1,
+                              kUdFew + kUnWarps}) {
+                    if (W > kUdFew && !few) continue;
                     const double ms = time_ms([&] { up_down<float>(down != 0, dp, l, T, (float*)(down ? b->U : b->Q),
                                                                    nrhs, down != 0, st, W); }, 5);
                     if (W == def) def_ms = ms;

@@ -787,13 +787,16 @@ int skel_test_set_updown(skel_handle h, int code) {
     return guarded([&] {
         if (!h) throw Error(SKEL_ERR_ARG, "handle is NULL");
         if (!h->dev) throw Error(SKEL_ERR_STATE, "plan was built host-only");
-        static const int ok[] = {0, 1, 2, 4, 8, 17, 18, 20, 24};
+        static const int ok[] = {0, 1, 2, 4, 8, 17, 18, 20, 24, 33, 40};
         bool valid = false;
         for (int c : ok) valid |= c == code;
-        if (!valid) throw Error(SKEL_ERR_ARG, "code must be 0, 1, 2, 4, 8, 17, 18, 20 or 24");
+        if (!valid) throw Error(SKEL_ERR_ARG, "code must be 0, 1, 2, 4, 8, 17, 18, 20, 24, 33 or 40");
         const int nl = (int)h->dev->up_level_ptr.size() - 1;
-        h->dev->ud_warps_up.assign(std::max(nl, 0), (int8_t)code);
-        h->dev->ud_warps_down.assign(std::max(nl, 0), (int8_t)code);
+        const int wide = code > 32 ? 0 : code;          // 33, 40: shapes of up to 8 right-hand sides only
+        h->dev->ud_warps_up.assign(std::max(nl, 0), (int8_t)wide);
+        h->dev->ud_warps_down.assign(std::max(nl, 0), (int8_t)wide);
+        h->dev->ud_few_up.assign(std::max(nl, 0), (int8_t)code);
+        h->dev->ud_few_down.assign(std::max(nl, 0), (int8_t)code);
     });
 }
 

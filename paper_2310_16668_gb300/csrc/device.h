@@ -99,6 +99,7 @@ struct DevicePlan {
     // FP32 up/down launch shape per level: warps per CTA (0: the default
     // rule), set by the autotuner
     std::vector<int8_t> ud_warps_up, ud_warps_down;
+    std::vector<int8_t> ud_few_up, ud_few_down;   // the same for up to kUnMaxRhs right-hand sides
     int tcs_stages = 4;                    // stages per CTA of the per-tile stored kernel (4 or 8)
     // tensor-core upward / downward passes (FP32_TC, real kernels): per
     // direction the work items (UdItem) grouped by level and their A blobs

@@ -4,27 +4,22 @@
 // (31 of 32 lanes idle at nrhs = 1, and FP64 multiply-adds cost the same for
 // idle lanes); here a lane owns an output row.
 //
-// A work-list entry is 32 output rows of one box. Its inner index is cut into
-// at most 8 segments (un_segment() long, from the box alone), whose partial
-// sums are added in order. W = 8: a CTA of 8 warps per entry, one per segment;
-// W = 1: 8 entries per CTA, each warp runs through its entry's segments, for
-// levels whose boxes have at most two (2D trees: 64 curve sets at 4 columns
-// took 0.19 ms a pass with a CTA per entry). Per inner index a warp loads one
-// coalesced column of 32 T entries (16 in flight) and the row's RT values from
-// a staged block. Every shape gives the same bits.
-// 64 curve sets, 4 right-hand sides, up + down per apply: 246 -> 209 us.
+// A work-list entry is 32 output rows of one box. As in those kernels the inner
+// index runs in chunks of 32, chunk ch in stream ch % 8 (for FP32 these are
+// their streams, and the bits are theirs: one more launch shape), and the
+// streams' sums are added in order. W = 8: a CTA of 8 warps per entry, a stream
+// per warp; W = 1: 8 entries per CTA, each warp runs through its entry's streams.
+// Per inner index a warp loads one coalesced column of 32 T entries and the row's
+// RT values from a staged block; the next group of T entries, the next chunk's
+// values and the entries after those are in flight while a group is multiplied.
 #pragma once
 
 #include "skel_kernels.cuh"
 
 namespace skel {
 
-constexpr int kUnWarps = 8;                // warps per CTA; segments of an entry, at most
+constexpr int kUnWarps = 8;                // warps per CTA; streams of an entry
 constexpr int kUnMaxRhs = 8;
-__host__ __device__ constexpr int un_segment(int ninner) {
-    const int eighth = ((ninner + 7) / 8 + 31) / 32 * 32;
-    return eighth > 64 ? eighth : 64;
-}
 
 template <class S, bool DOWN, int RT, int W>
 __global__ void __launch_bounds__(32 * kUnWarps) updown_narrow_kernel(const UpBox* __restrict__ up,
@@ -52,27 +47,41 @@ __global__ void __launch_bounds__(32 * kUnWarps) updown_narrow_kernel(const UpBo
     }
     if (row0 >= nout) return;
     const bool rowok = row0 + lane < nout;
-    const int seg = un_segment(ninner), nseg = (ninner + seg - 1) / seg;
+    const int nch = (ninner + 31) / 32, nst = nch < kUnWarps ? nch : kUnWarps;
     const S* Tr = T + u.T_off + row0 + lane;
-    S acc[RT], tot[RT];
+    constexpr int G = sizeof(S) <= 4 ? 16 : sizeof(S) <= 8 ? 8 : 4;   // T entries of a group
+    // inner indices j0 .. j0 + G - 1 of this lane's row
+    auto load_t = [&](int j0, S* a) {
+#pragma unroll
+        for (int q = 0; q < G; ++q) a[q] = rowok && j0 + q < ninner ? Tr[(int64_t)(j0 + q) * nout] : zero<S>();
+    };
+    // this lane's inner index of chunk ch: its entry, and its values
+    auto entry_of = [&](int ch) -> int64_t {
+        const int j = 32 * ch + lane;
+        if (j >= ninner) return -1;
+        return DOWN ? u.dst + j : u.off + pos[u.off + k + j];
+    };
+    auto load_x = [&](int64_t e, S* x) {
+#pragma unroll
+        for (int c = 0; c < RT; ++c) x[c] = e >= 0 && c < nrhs ? X[e * nrhs + c] : zero<S>();
+    };
+    S acc[RT], tot[RT], x[RT], a[G], b[G];
 #pragma unroll
     for (int c = 0; c < RT; ++c) acc[c] = tot[c] = zero<S>();
-    for (int sg = W > 1 ? warp : 0; sg < nseg; sg += W) {
-        const int j_hi = min((sg + 1) * seg, ninner);
-        for (int j0 = sg * seg; j0 < j_hi; j0 += 32) {
-            const int jn = min(32, j_hi - j0);
-            if (lane < jn) {
-                const int64_t e = DOWN ? u.dst + j0 + lane : u.off + pos[u.off + k + j0 + lane];
+    for (int st = W > 1 ? warp : 0; st < nst; st += W) {
+        load_t(32 * st, a);
+        load_x(entry_of(st), x);
+        int64_t next = entry_of(st + kUnWarps);
+        for (int ch = st; ch < nch; ch += kUnWarps) {
+            const int jn = min(32, ninner - 32 * ch);
 #pragma unroll
-                for (int c = 0; c < RT; ++c) sq[warp][lane][c] = c < nrhs ? X[e * nrhs + c] : zero<S>();
-            }
+            for (int c = 0; c < RT; ++c) sq[warp][lane][c] = x[c];
             __syncwarp();
-            constexpr int G = 16;
-            for (int g0 = 0; g0 < jn; g0 += G) {
-                S a[G];
+            load_x(next, x);
+            next = entry_of(ch + 2 * kUnWarps);
 #pragma unroll
-                for (int q = 0; q < G; ++q)
-                    a[q] = rowok && g0 + q < jn ? Tr[(int64_t)(j0 + g0 + q) * nout] : zero<S>();
+            for (int g0 = 0; g0 < 32; g0 += G) {
+                load_t(g0 + G < 32 ? 32 * ch + g0 + G : 32 * (ch + kUnWarps), b);
 #pragma unroll
                 for (int q = 0; q < G; ++q)
                     if (g0 + q < jn) {
@@ -80,13 +89,15 @@ __global__ void __launch_bounds__(32 * kUnWarps) updown_narrow_kernel(const UpBo
 #pragma unroll
                         for (int c = 0; c < RT; ++c) acc[c] += v * sq[warp][g0 + q][c];
                     }
+#pragma unroll
+                for (int q = 0; q < G; ++q) a[q] = b[q];
             }
             __syncwarp();
         }
         if constexpr (W == 1) {
 #pragma unroll
             for (int c = 0; c < RT; ++c) {
-                tot[c] = sg == 0 ? acc[c] : tot[c] + acc[c];
+                tot[c] = st == 0 ? acc[c] : tot[c] + acc[c];
                 acc[c] = zero<S>();
             }
         }
@@ -105,8 +116,8 @@ __global__ void __launch_bounds__(32 * kUnWarps) updown_narrow_kernel(const UpBo
         for (int i = threadIdx.x; i < 32 * nrhs; i += 32 * W) {
             const int row = i / nrhs, c = i - row * nrhs, orow = row0 + row;
             if (orow >= nout) continue;
-            S v = nseg > 0 ? ps[0][c][row] : zero<S>();
-            for (int q = 1; q < nseg; ++q) v = v + ps[q][c][row];
+            S v = nst > 0 ? ps[0][c][row] : zero<S>();
+            for (int q = 1; q < nst; ++q) v = v + ps[q][c][row];
             const int64_t src = row_at(orow) + c, dst = DOWN ? src : (u.dst + orow) * nrhs + c;
             X[dst] = X[src] + v;
         }

@@ -178,16 +178,21 @@ struct TcItem {                         // 64 bytes
 static_assert(sizeof(TcItem) == 64, "TcItem layout");
 
 // log2 of the tiles of a segment, the shortest piece into which the on-the-fly
-// kernel can cut an item's list: 128 tiles, and 16 where a 3D plan has so few
-// that its lists (about 60 tiles) would each be one piece and leave most of the
-// chip idle. Near kernel, 32 right-hand sides, leaves of 128, segments of 128, 32
-// and 16 (and one item per CTA, two threads per row, before): N = 1,500 46, 43, 29
-// (42) us, 3,000 79, 43, 38 (69), 5,000 119, 56, 60 (103), 7,000 (12,187 tiles)
-// 124, 90, 82. From N = 8,000 (18,077 tiles) segments of 128 are faster than that
-// kernel (131, 137) and leave larger plans fewer sums to add up. Fixed with the item, so that a
-// merged plan gives each set its own plan's sums.
-constexpr int64_t kShortTiles = 14592;  // 24 for each of the 608 groups of rows that run at a time
-constexpr int tc_segment(int dim, int64_t tiles) { return dim == 3 && tiles < kShortTiles ? 4 : 7; }
+// kernel can cut an item's list: 128 tiles, and 16 or 32 where a 3D plan has so
+// few that its lists (60 to 130 tiles) would each be about one piece and leave
+// part of the chip idle. Near kernel, 32 right-hand sides, leaves of 128, segments
+// of 128, 32 and 16 (and the kernel with one item per CTA and two threads per
+// row that it replaced), us: N = 1,500 46, 43, 29 (42); 3,000 79, 43, 38 (69);
+// 5,000 119, 56, 60 (103); 8,000 131, 93, 100 (138); 16,000 189, 152, 154 (183);
+// 20,011 212, 194, 208 (240); leaves of 40, N = 20,000 303, 256, 278 (273);
+// sphere + cluster, N = 40,000 211, 200, 199 (200). From N = 28,000 (89,221 tiles)
+// 32 and 128 are alike (320), and longer segments are fewer sums to add up.
+// Fixed with the item, so that a merged plan gives each set its own plan's sums.
+constexpr int64_t kShortTiles = 14592;  // 16 tiles: up to 24 for each of the 608 groups of rows that run at a time
+constexpr int64_t kMidTiles = 80000;    // 32 tiles
+constexpr int tc_segment(int dim, int64_t tiles) {
+    return dim != 3 || tiles >= kMidTiles ? 7 : tiles >= kShortTiles ? 5 : 4;
+}
 
 struct Layout {
     int threads = 0;                    // host threads of its builders (0 = all, 1 = the caller's only)

@@ -381,6 +381,22 @@ __global__ void __launch_bounds__(256) tc_bprep_kernel(const int64_t* __restrict
     }
 }
 
+// U[row][r0 + c0 ..] = v
+template <int NC>
+__device__ __forceinline__ void tc_put_rows(const TcArgs& a, int64_t row, int c0, const float* v) {
+    float* u = a.U + row * a.nrhs + a.r0 + c0;
+    const int left = a.nrhs - a.r0 - c0;
+    if (a.nrhs % 4 == 0 && left >= NC) {
+        float4* u4 = reinterpret_cast<float4*>(u);
+#pragma unroll
+        for (int c = 0; c < NC / 4; ++c) u4[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (c < left) u[c] = v[c];
+    }
+}
+
 // U[row][r0 + c0 ..] = scale * v (the first segment of an item) or += it: a
 // row has one writer, so its segments add up in order
 template <int KIND, int NC>
@@ -437,14 +453,14 @@ __device__ __forceinline__ int tile_word(uint32_t qm, int quad, int row, int nro
 // tc_near_kernel, so both give the same result bit for bit. Bound: HBM,
 // nrows x 128 bytes of kernel values per tile.
 static_assert(kSrcPerThread == 16, "stored tiles assume two compute threads per row");
-// Tensor memory: D0, D1 [0, 64) for the pairs in turn, L [64, 96), A[b] hi at
-// 128 + 64 b, lo at 160 + 64 b (b < 2). Two A buffers suffice: the buffer of
+// Tensor memory: D0, D1 [0, 64) for the pairs in turn, L [64, 96), the sum of
+// the finished segments [96, 128), A[b] hi at 128 + 64 b, lo at 160 + 64 b (b < 2). Two A buffers suffice: the buffer of
 // tile u was last read by MMA(u - 2), which has been waited for before tile u
 // is written.
 // NST data stages (24 KB each): 4 with two CTAs per SM, or 8 with one CTA
 // per SM (the autotuner times both).
 constexpr int kNAS = 2;                        // A buffers
-constexpr uint32_t kColSL = 64, kColSA = 128;
+constexpr uint32_t kColSL = 64, kColSOuter = 96, kColSA = 128;
 
 // The stored kernels' MMAs of tile m (its B operand at bh): the sum of
 // tc_near.cuh, with pair p's hi*hi products in D[p % 2]; mask: tiles of a
@@ -493,6 +509,32 @@ struct TcSums {
         clear();
     }
 };
+// A finished segment, scaled, is added to those before it in tensor memory (the
+// additions of tc_add_rows); the last one takes the sum to U. Reading and
+// writing U at every segment cost segments of 32 tiles 4% (N = 12,000, 32
+// right-hand sides, one pass: 118 us, here 113).
+template <int KIND, int NC>
+__device__ __forceinline__ void tcs_segment(const TcArgs& a, uint32_t ocol, int64_t row, bool valid, int c0, bool first,
+                                            bool last, float* v) {
+    const float scale = (float)green_scale<KIND>();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) v[c] = __fmul_rn(scale, v[c]);
+    if (!first) {
+        uint32_t o[NC];
+        tmem_ld16(ocol, o);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = __fadd_rn(__uint_as_float(o[c]), v[c]);
+    }
+    if (!last) {
+        uint32_t o[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) o[c] = __float_as_uint(v[c]);
+        tmem_st16(ocol, o);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    } else if (valid) {
+        tc_put_rows<NC>(a, row, c0, v);
+    }
+}
 struct alignas(128) TcTileStage {
     float b[2 * 1024];                         // B hi, B lo (the first 8 KB of the chunk block)
     float4 ga[kTileFloats / 4];                // the tile's kept quads
@@ -603,13 +645,13 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
             if (!mbar_wait(sm_addr(&S.empty[m % NST]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         };
-        // the segment that ends before tile u goes to U
+        // the segment that ends before tile u
         auto flush = [&](int u) {
             if (u > 0) done(u - 1);
             const int s0 = u > 0 ? (u - 1) & ~mask : 0;
             float v[kCols];
             sums.finish(tcol, u - s0, v);
-            if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
+            tcs_segment<KIND, kCols>(a, tcol + kColSOuter, row_off + row, valid, kCols * half, s0 == 0, u == ntile, v);
         };
         const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
         for (int u = 0; u < ntile; ++u) {

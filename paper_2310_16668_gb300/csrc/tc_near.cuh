@@ -24,7 +24,7 @@
 // 66 -> 43.
 //
 // The sum, the same for all forms and for the stored kernels (so all give
-// the same bits): an item's tile list is cut into segments of 128 tiles (16 in small 3D plans, tc_segment)
+// the same bits): an item's tile list is cut into segments of 128 tiles (16 or 32 in small 3D plans, tc_segment)
 // and a segment into pairs of tiles. The hi*hi products of a pair accumulate in
 // tensor memory (D: 8 K-steps) and are then added to an FP32 register sum;
 // the hi*lo and lo*hi products of the whole segment accumulate in a second

@@ -143,13 +143,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
             if (!mbar_wait(sm_addr(&S.emptyB[m % NB]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         };
-        // the segment that ends before tile u goes to U
+        // the segment that ends before tile u
         auto flush = [&](int u) {
             if (u > 0) done(u - 1);
             const int s0 = u > 0 ? (u - 1) & ~mask : 0;
             float v[kCols];
             sums.finish(tcol, u - s0, v);
-            if (valid) tc_add_rows<KIND, kCols>(a, row_off + row, kCols * half, s0 > 0, v);
+            tcs_segment<KIND, kCols>(a, tcol + kColSOuter, row_off + row, valid, kCols * half, s0 == 0, u == ntile, v);
         };
         const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
         for (int u = 0; u < ntile; ++u) {

@@ -80,7 +80,9 @@ def test_merged_plans_keep_their_sets_segments():
 
 @pytest.mark.parametrize("kind,n,leaf,form", [
     ("laplace3d", 30000, 128, "pairs, cut"),
-    ("laplace3d", 16500, 16500, "pairs, cut"),           # one leaf: 129 items, the last one of 116 rows
+    ("laplace3d", 20000, 20000, "pairs, cut"),           # one leaf: 157 items, the last one of 32 rows
+    ("laplace3d", 20011, 128, "pairs, pieces of 32"),
+    ("laplace3d", 12000, 128, "single, pieces of 32"),
     ("laplace3d", 120000, 128, "pieces of two segments"),
     ("laplace3d", 150000, 128, "pairs, whole lists"),    # the form of every larger 3D plan
     ("laplace2d", 4300, 4300, "single, cut"),
@@ -92,10 +94,13 @@ def test_forms_match_fp64(kind, n, leaf, form, nrhs):
     un = _units(f)
     if form.startswith("single"):
         assert un["single"] > 0 and un["cut"] > 0 and un["shared"] == un["unrelated"] == 0
+        assert un["longest"] == (32 if "32" in form else 128)
     else:
         assert un["shared"] > 0 and un["unrelated"] > 0
         if form == "pairs, cut":
             assert un["cut"] > 0 and un["longest"] == 128
+        elif form == "pairs, pieces of 32":
+            assert un["cut"] > 0 and un["longest"] == 32
         elif form == "pieces of two segments":
             assert un["cut"] > 0 and un["longest"] == 256
         else:

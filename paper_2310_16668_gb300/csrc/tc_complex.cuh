@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(kThreadsC, 1) tc_cnear_kernel(const TcArgs a) 
                 if (cut) tc_ceval<false, true>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
                 else tc_ceval<false, false>(st.xh + j0, nt, nl, a.kappa, kb, grh, grl, gih, gil);
             }
+            __syncwarp();
             const int g = u & (kTcOuter - 1);                  // tile of the group
             if (u > 0 && g == 0) {
                 flush(u, u - kTcOuter);

@@ -161,6 +161,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     }
 }
 
+// The same for a whole warp. Every lane polls (and gives up) by itself, so the
+// lanes may leave the wait apart: they come together before the tensor-memory
+// instructions that follow, which a warp executes as one (.sync.aligned).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+    const bool ok = mbar_wait(bar, parity, limit_ns);
+    __syncwarp();
+    return ok;
+}
+
 // An early look at a barrier whose phase is needed later: a wait takes 150 to
 // 300 clocks of a busy SM even when the phase is complete, so it is asked for
 // before work that does not need it and settled after that work.
@@ -172,7 +181,7 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
 }
 __device__ __forceinline__ bool mbar_settle(uint32_t early, uint32_t bar, uint32_t parity, uint64_t limit_ns) {
     bool ok = true;
-    if (!__all_sync(0xffffffffu, early != 0u)) ok = mbar_wait(bar, parity, limit_ns);
+    if (!__all_sync(0xffffffffu, early != 0u)) ok = mbar_wait_warp(bar, parity, limit_ns);
     asm volatile("" ::: "memory");
     return ok;
 }
@@ -642,7 +651,7 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
         sums.clear();
         // wait for tile m's MMAs
         auto done = [&](int m) {
-            if (!mbar_wait(sm_addr(&S.empty[m % NST]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
+            if (!mbar_wait_warp(sm_addr(&S.empty[m % NST]), (uint32_t)((m / NST) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         };
         // the segment that ends before tile u
@@ -683,6 +692,7 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
                 flush(u);
             } else {
                 if (u >= 2) done(u - 2);
+                else __syncwarp();                             // (after the wait for the copies)
                 // before the pair that starts with tile u, the pair two before it
                 if (!(u & 1) && (u & mask) >= 4) sums.pair(tcol, ((u & mask) >> 1) - 2);
             }
@@ -901,7 +911,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_sym_kernel(const TcArgs a) {
             S.outer[c][tid] = 0.f;
         }
         auto drain = [&](int mm) {
-            if (!mbar_wait(sm_addr(&S.empty[mm % kNSY]), (uint32_t)((mm / kNSY) & 1), a.wait_ns)) err = true;
+            if (!mbar_wait_warp(sm_addr(&S.empty[mm % kNSY]), (uint32_t)((mm / kNSY) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             uint32_t v[kCols];
             tmem_ld16(tbase + lane_off + kColD + 32u * (mm & 1) + (uint32_t)(kCols * half), v);
@@ -918,7 +928,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_sym_kernel(const TcArgs a) {
         const float2 m1 = make_float2(-1.f, -1.f), split = make_float2(8193.f, 8193.f);
         for (int u = 0; u < ntile; ++u) {
             const int s = u % kNSY;
-            const bool landed = mbar_wait(sm_addr(&S.full[s]), (uint32_t)((u / kNSY) & 1), a.wait_ns);
+            const bool landed = mbar_wait_warp(sm_addr(&S.full[s]), (uint32_t)((u / kNSY) & 1), a.wait_ns);
             if (!landed) err = true;
             const TcSymStage& st = S.st[s];
             // the row's kept sources of this tile, and where its block sits
@@ -959,6 +969,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_sym_kernel(const TcArgs a) {
             }
             if (u >= 2) drain(u - 2);
             const uint32_t acol = tbase + lane_off + kColA + 64u * (u % kNA) + (uint32_t)j0;
+            __syncwarp();
             tmem_st16(acol, ghi);
             tmem_st16(acol + 32u, glo);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");

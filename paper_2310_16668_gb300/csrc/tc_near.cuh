@@ -75,6 +75,29 @@ struct TcNearShared {
 constexpr int kNearSmemRequest = 113 * 1024;   // two CTAs (2 x 256 TMEM columns) per SM
 static_assert(sizeof(TcNearShared) <= kNearSmemRequest, "shared memory plan");
 
+// Alignment of every access wider than 4 bytes (an unaligned one is a fault):
+//   bulk copies, 16 bytes at both ends and in size: chunks start kChunkFloats
+//     apart in a.B and in a stage, descriptors 64 bytes apart in a.tiles and in
+//     tile[]; stages are 128-byte multiples of the shared memory's base;
+//   mbarriers, 8 bytes: uint64_t members behind whole stages;
+//   float4 reads of a chunk's coordinates: 2048 floats into the chunk, axes 32
+//     floats apart, lo parts 96, sources in steps of 8, 4 per read (16 of a
+//     tile's 32 sources per group: a multiple of 16 floats);
+//   float4 of a.X, a.Xlo: arrays of float4;
+//   float4 of U: only if nrhs is a multiple of 4, from columns that are
+//     multiples of 16 (r0 of 32);
+//   float4 of parts: rows of 32 floats, columns as for U;
+//   float4 of stored values (fill): an item starts at abase, a multiple of 4
+//     floats, and tiles are whole float4;
+//   tensor-memory columns are multiples of 8, and whole warps execute every
+//     tcgen05.st / ld (the waits before them end per thread: __syncwarp).
+// Nothing here depends on data a bounded wait could leave stale: after one gives
+// up, a descriptor may be wrong, but it only chooses among masks and flags.
+static_assert(sizeof(TcPairStage) % 128 == 0 && offsetof(TcPairStage, tile) % 16 == 0, "stage layout");
+static_assert(offsetof(TcNearShared, full) % 8 == 0 && offsetof(TcNearShared, tmem) % 4 == 0, "barriers");
+static_assert(kChunkFloats % 4 == 0 && (2048 + 96) % 4 == 0 && sizeof(SrcTile) == 64, "chunk layout");
+static_assert(sizeof(float) * kTcN % 16 == 0, "rows of partial sums");
+
 // log of 8 squared distances. Normal arguments: x = 2^e m with m in
 // [sqrt(1/2), sqrt(2)), f = m - 1 and log x = e ln 2 + (f - f^2/2 + f^3 P(f)),
 // P of degree 7 fitted to the series (relative error 6e-9), ln 2 as a sum of
@@ -322,10 +345,10 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
         if constexpr (SPLIT) {
             if (cnt >= back) {
                 const uint32_t t = cnt - back;
-                ok &= mbar_wait(sm_addr(&S.done[t & 1u][0]), (t >> 1) & 1u, a.wait_ns);
+                ok &= mbar_wait_warp(sm_addr(&S.done[t & 1u][0]), (t >> 1) & 1u, a.wait_ns);
             }
         } else {
-            if (cnt > 0u) ok &= mbar_wait(sm_addr(&S.done[g][b]), (cnt - 1u) & 1u, a.wait_ns);
+            if (cnt > 0u) ok &= mbar_wait_warp(sm_addr(&S.done[g][b]), (cnt - 1u) & 1u, a.wait_ns);
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
@@ -348,13 +371,14 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
         const int send = min(s0 + (1 << lseg), t_hi);
 #pragma unroll
         for (int c = 0; c < NC / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+        __syncwarp();                                      // (rows that are not valid skipped the end of a segment)
         tmem_zero<NC>(dcol);
         tmem_zero<NC>(lcol);
         if (SPLIT) tmem_zero<NC>(dcol + kColSplitD1);
         for (int t = s0; t < send; ++t) {
             const int ti = t & 1;
             const TcPairStage& st = S.st[ring + s];
-            if (ti == 0) ok &= mbar_wait(sm_addr(&S.full[ring + s]), ph, a.wait_ns);
+            if (ti == 0) ok &= mbar_wait_warp(sm_addr(&S.full[ring + s]), ph, a.wait_ns);
             const SrcTile& tl = st.tile[ti];
             const float* xs = st.chunk[ti] + 2048;
             // touching leaves take the form with lo parts and guards, and so do
@@ -429,10 +453,7 @@ __device__ __forceinline__ bool tc_near_rows(const TcArgs& a, TcNearShared& S, i
                                         dst[tile_word(qm, 2 * tq + h, row, nrows)] =
                                             make_float4(gv[4 * h], gv[4 * h + 1], gv[4 * h + 2], gv[4 * h + 3]);
                             }
-                            if (e == 0) {
-                                wait_done(b, 2u);
-                                __syncwarp();
-                            }
+                            if (e == 0) wait_done(b, 2u);
                             tc_split_store(gv, at_col + 32u * b + 8u * e);
                         }
                         if (b == 0) drain();

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
         sums.clear();
         // wait for tile m's MMAs
         auto done = [&](int m) {
-            if (!mbar_wait(sm_addr(&S.emptyB[m % NB]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
+            if (!mbar_wait_warp(sm_addr(&S.emptyB[m % NB]), (uint32_t)((m / NB) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         };
         // the segment that ends before tile u
@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_stored_ring_kernel(const TcA
                 flush(u);
             } else {
                 if (u >= 2) done(u - 2);
+                else __syncwarp();                             // (after the wait for the copies)
                 // before the pair that starts with tile u, the pair two before it
                 if (!(u & 1) && (u & mask) >= 4) sums.pair(tcol, ((u & mask) >> 1) - 2);
             }

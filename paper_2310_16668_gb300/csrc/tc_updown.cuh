@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_ud_kernel(const UdArgs a) {
 #pragma unroll
         for (int c = 0; c < 16; ++c) acc[c] = 0.f;
         auto drain = [&](int m) {                            // add tile m's product (its MMAs are done)
-            if (!mbar_wait(sm_addr(&S.empty[m % kUdNST]), (uint32_t)((m / kUdNST) & 1), a.wait_ns)) err = true;
+            if (!mbar_wait_warp(sm_addr(&S.empty[m % kUdNST]), (uint32_t)((m / kUdNST) & 1), a.wait_ns)) err = true;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             uint32_t v[16];
             tmem_ld16(tbase + lane_off + kColD + 32u * (m & 1) + 16u * half, v);
@@ -209,14 +209,14 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_ud_kernel(const UdArgs a) {
         };
         float xc[4] = {0.f, 0.f, 0.f, 0.f}, xn[4] = {0.f, 0.f, 0.f, 0.f};
         if (ntile > 0) {
-            if (!mbar_wait(sm_addr(&S.full[0]), 0u, a.wait_ns)) err = true;
+            if (!mbar_wait_warp(sm_addr(&S.full[0]), 0u, a.wait_ns)) err = true;
             load_b(0, xc);
         }
         for (int t = 0; t < ntile; ++t) {
             const int s = t % kUdNST;
             // the next tile's B rows go out now and arrive while this one is processed
             if (t + 1 < ntile) {
-                if (!mbar_wait(sm_addr(&S.full[(t + 1) % kUdNST]), (uint32_t)(((t + 1) / kUdNST) & 1), a.wait_ns))
+                if (!mbar_wait_warp(sm_addr(&S.full[(t + 1) % kUdNST]), (uint32_t)(((t + 1) / kUdNST) & 1), a.wait_ns))
                     err = true;
                 load_b(t + 1, xn);
             }
@@ -251,6 +251,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_ud_kernel(const UdArgs a) {
             // A buffer and accumulator t & 1 were last used by tile t - 2
             if (t >= 2) drain(t - 2);
             const uint32_t acol = tbase + lane_off + kUdColA + 96u * (t & 1) + 16u * half;
+            __syncwarp();
             tmem_st16(acol, gh);
             tmem_st16(acol + 32u, gm);
             tmem_st16(acol + 64u, gl);

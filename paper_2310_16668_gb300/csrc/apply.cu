@@ -857,7 +857,6 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
     cudaFree(units);
 }
 
-
 // The on-the-fly kernel's units, longest first. Two items with consecutive
 // rows of one box share a CTA and the tiles it copies, the others pair up by
 // the length of their lists: the CTA's groups then evaluate 32 values a thread
@@ -870,7 +869,12 @@ void fill_tiles(DevicePlan* dp, cudaStream_t st, int mode) {
 // (TcItem::lseg); tc_segments_kernel adds the segments of a cut item.
 // Neither pairing nor cutting changes a result.
 constexpr int64_t kPairShare = 16;             // share from which 3D items share CTAs
-constexpr int64_t kCutShare = 256;             // ... up to which long lists are cut
+// ... up to which long lists are cut. Near kernel, cut against whole: N = 30,000
+// (share 39) 319, 474 us; 60,000 (93) 635, 799; 90,000 (165) 1051, 1025; 120,000
+// (202) 1303, 1291; 150,000 (288) 1772, 1757; 262,144 3314, 3296: the lists are
+// long against the CTAs' share up to about 128, and between 128 and 256 cutting
+// costs 1 to 2.5%
+constexpr int64_t kCutShare = 256;
 struct Units {
     std::vector<TcUnit> units;
     std::vector<int64_t> part0;                            // per item (see TcArgs)

@@ -1,10 +1,10 @@
 // Translations on the CUDA cores with every kernel value used twice: the
 // kernels are symmetric (complex-symmetric for Helmholtz) and so is the set of
 // pairs the translations evaluate, so G(t, s) serves u_t += G q_s and
-// u_s += G q_t. For FP64, where the evaluation is the cost: GB300 issues 2 FP64
-// lanes per SM and clock, and a value of 3D Laplace takes 11 FP64 operations,
-// so an interaction with one right-hand side takes 6.5 here and 12 in
-// near_kernel.
+// u_s += G q_t. For FP64, where the evaluation is the cost: GB300 issues 1.66 FP64
+// lanes per SM and clock (measured), and a value of 3D Laplace takes 11 FP64
+// operations, so an interaction with one right-hand side takes 6.5 here and 12
+// in near_kernel.
 //
 // A warp owns an item: one target chunk (up to 32 entries of a box, one per
 // lane) against up to sym_chunks() source chunks of one box (each unordered
@@ -45,8 +45,9 @@ struct SymArgs {
 // ---- natural logarithm of a positive normal double ---------------------------------
 // Table-driven (P.T.P. Tang, "Table-driven implementation of the logarithm
 // function in IEEE arithmetic", ACM TOMS 16, 1990): x = 2^e z with
-// z in [sqrt(1/2), sqrt(2)), c the table's point near z (an exact short
-// reciprocal 1/c is stored), f = z / c - 1 from one FMA, |f| < 2^-8, and
+// z in [sqrt(1/2), sqrt(2)), c the table's point near z (the double 1/c is stored
+// and log c is that of its exact reciprocal), f = z / c - 1 from one FMA,
+// |f| < 2^-8, and
 // log x = e ln 2 + log c + log1p(f) with a degree-6 series; ln 2 and log c are
 // sums of a multiple of 2^-40 and a rest, so that e ln 2 + log c loses nothing.
 // 13 FP64 operations (the CUDA library's log takes the time of about 27).

@@ -10,9 +10,10 @@
 // swizzle, 8 x 16-byte core matrices), split into TF32 hi and lo, followed by
 // the chunk's coordinates. tc_near.cuh evaluates the kernel and multiplies; this
 // file holds what the tensor-core kernels share and the kernels that read
-// stored values. All of them form the same sum (tc_near.cuh states it) and so
-// give the same bits. The dropped lo*lo term and the truncation of the lo parts
-// are below 2^-21 of each product.
+// stored values. The on-the-fly kernel and the two kernels of the per-tile store
+// (here and in tc_stored_ring.cuh) form the same sum (tc_near.cuh states it) and
+// so give the same bits; the symmetric store's has a sum of its own. The dropped
+// lo*lo term and the truncation of the lo parts are below 2^-21 of each product.
 //
 // Masks: a source that a target row's slot must skip (the regrouped
 // subtractions of Algorithm 2) gets G = 0 in that row.
@@ -450,22 +451,22 @@ __device__ __forceinline__ int tile_word(uint32_t qm, int quad, int row, int nro
 // ---------------------------------------------------------------------------
 // Stored-operator mode, per-tile store: the same translations with every
 // tile's kernel values read from the tiles the fill pass (tc_near_kernel with
-// REC = kRecTiles) wrote, instead of evaluated. Tile u of an item with nrows
-// rows keeps its nrows x 32 values (unscaled FP32, zero where a row's slot
-// skips the source) at A + abase[item] + u * nrows * 32, ordered so that
-// compute thread (row, half) reads its 16 values as four 16-byte words with
-// consecutive rows adjacent: value (row, j = 16 half + 4 q + e) at
-// ((half * 4 + q) * nrows + row) * 4 + e. Per tile the producer copies 24 KB
-// at most (the chunk's B hi + lo and the kernel tile); the compute warps only
-// split the values into TF32 hi + lo and write A to tensor memory. The MMA
-// issue, the accumulator drain and the two-level sum are those of
-// tc_near_kernel, so both give the same result bit for bit. Bound: HBM,
-// nrows x 128 bytes of kernel values per tile.
+// REC = kRecTiles) wrote, instead of evaluated. A tile of an item with nrows rows
+// keeps the quads (4 consecutive sources) in which some row keeps a source (its
+// byte of qmask): unscaled FP32, zero where a row's slot skips the source. An
+// item's tiles lie back to back from A + abase[item]; a kept quad is nrows
+// 16-byte words, quads in order (tile_word), so that consecutive rows are
+// adjacent. Per tile the producer copies 24 KB at most (the chunk's B hi + lo and
+// the kept quads); the compute warps only split the values into TF32 hi + lo and
+// write A to tensor memory, zeros for the other quads. The sum is that of
+// tc_near_kernel, so both give the same result bit for bit. Bound: HBM, 16 bytes
+// per row and kept quad: 12.35 ms and 78.7 GB at N = 2^20, 0.96 of the copy
+// bandwidth.
 static_assert(kSrcPerThread == 16, "stored tiles assume two compute threads per row");
 // Tensor memory: D0, D1 [0, 64) for the pairs in turn, L [64, 96), the sum of
-// the finished segments [96, 128), A[b] hi at 128 + 64 b, lo at 160 + 64 b (b < 2). Two A buffers suffice: the buffer of
-// tile u was last read by MMA(u - 2), which has been waited for before tile u
-// is written.
+// the finished segments [96, 128), A[b] hi at 128 + 64 b, lo at 160 + 64 b
+// (b < 2). Two A buffers suffice: the buffer of tile u was last read by
+// MMA(u - 2), which has been waited for before tile u is written.
 // NST data stages (24 KB each): 4 with two CTAs per SM, or 8 with one CTA
 // per SM (the autotuner times both).
 constexpr int kNAS = 2;                        // A buffers
@@ -724,9 +725,11 @@ __global__ void __launch_bounds__(kTcThreads, NST <= 4 ? 2 : 1) tc_stored_kernel
 // fixed per-stage areas would). The compute warps find their row chunk's
 // block from the ring base the producer recorded and the sizes of the blocks
 // before it, read their row's 16 values directly or transposed, apply the
-// row's keep mask, split into TF32 hi + lo and write A to tensor memory. The
-// MMA issue, the accumulator drain and the two-level sum are those of
-// tc_near_kernel. Bound: HBM, 4 bytes per stored value.
+// row's keep mask, split into TF32 hi + lo and write A to tensor memory. Its sum
+// is its own: the 12 MMAs of a tile (hi*hi, hi*lo, lo*hi) go into one accumulator
+// of two in turn, every tile is added to FP32 register sums, and those of
+// kTcOuter tiles to outer sums in shared memory (error 3.6e-7 where the
+// on-the-fly kernel's is 2.1e-7). Bound: HBM, 4 bytes per stored value.
 static_assert(kSrcPerThread == 16, "stored tiles assume two compute threads per row");
 constexpr int kNSY = 6;                        // stages (B operand, descriptors)
 constexpr int kRing = 10240;                   // floats of the block ring (40 KB)

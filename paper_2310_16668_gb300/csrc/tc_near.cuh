@@ -19,13 +19,14 @@
 // left of the hand-overs. FP32, 32 right-hand sides, before (one item per CTA,
 // two threads per row, three accumulating MMAs per K-step) and after: 3D,
 // leaves of 128, N = 65,536 922 -> 777 us, 262,144 3988 -> 3290 us, 20,011
-// 241 -> 211, 12,000 167 -> 136, 3,000 69 -> 79 (a segment of 128 tiles is the
-// shortest piece of a list); 2D, leaves of 64, N = 65,536 252 -> 218, 3,000
-// 66 -> 43.
+// 240 -> 195, 12,000 166 -> 131, 3,000 69 -> 38; 2D, leaves of 64, N = 65,536
+// 252 -> 212, 3,000 66 -> 43. Plans of up to 500 points with few right-hand sides
+// take up to 2 us more (N = 300, 4 right-hand sides, apply 28.7 -> 30.7).
 //
-// The sum, the same for all forms and for the stored kernels (so all give
-// the same bits): an item's tile list is cut into segments of 128 tiles (16 or 32 in small 3D plans, tc_segment)
-// and a segment into pairs of tiles. The hi*hi products of a pair accumulate in
+// The sum, the same for all forms and for the kernels of the per-tile store (so
+// all give the same bits): an item's tile list is cut into segments of 128 tiles
+// (16 or 32 in small 3D plans, tc_segment) and a segment into pairs of tiles. The
+// hi*hi products of a pair accumulate in
 // tensor memory (D: 8 K-steps) and are then added to an FP32 register sum;
 // the hi*lo and lo*hi products of the whole segment accumulate in a second
 // accumulator (L), which is 2^-11 of the first in size, so that its rounding
@@ -100,8 +101,11 @@ static_assert(sizeof(float) * kTcN % 16 == 0, "rows of partial sums");
 
 // log of 8 squared distances. Normal arguments: x = 2^e m with m in
 // [sqrt(1/2), sqrt(2)), f = m - 1 and log x = e ln 2 + (f - f^2/2 + f^3 P(f)),
-// P of degree 7 fitted to the series (relative error 6e-9), ln 2 as a sum of
-// two floats the first of which has 9 significant bits: within 0.9 ulp, half
+// the argument reduction of S. Moshier's logf (Cephes), here by the exponent bits
+// relative to those of sqrt(1/2); P of degree 7 fitted to
+// (log(1 + f) - f + f^2/2) / f^3 on that interval (against 64 bits: within 8e-9 of
+// the logarithm), ln 2 as a sum of two floats the first of which has 9
+// significant bits (as there): within 0.9 ulp, half
 // the instructions of logf because two values share each. on: 1, or 0 for a row
 // that keeps none of these sources. ADJ: subnormal x (whose exponent field says
 // nothing) go to logf; 0 for x = 0 if the leaves touch.

@@ -12,6 +12,12 @@
 // Per inner index a warp loads one coalesced column of 32 T entries and the row's
 // RT values from a staged block; the next group of T entries, the next chunk's
 // values and the entries after those are in flight while a group is multiplied.
+// Latency-bound on small levels (about 6 us a launch), by the loads of T on large
+// ones. FP32, 1 and 4 right-hand sides, the best column-per-lane shape against
+// this kernel: 64 boxes of 174 x 797, up 42, 42 -> 12, 15 us, down 29, 26 -> 14, 17;
+// 4,096 boxes of 21 x 47, up 27, 20 -> 11, 14, down 28, 26 -> 10, 15. Whole applies:
+// 3D N = 65,536, one column, 595 -> 504 us; 2D N = 200,000, 4 columns, 845 -> 641;
+// sphere + cluster N = 22,894, 4 columns, tuned, 217 -> 171.
 #pragma once
 
 #include "skel_kernels.cuh"

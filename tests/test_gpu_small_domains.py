@@ -45,7 +45,7 @@ def _rounding(x):
     return worst / (4 * math.pi)
 
 
-@pytest.mark.parametrize("form", ["on the fly", "stored", "merged"])
+@pytest.mark.parametrize("form", ["on the fly", "stored", "symmetric", "merged"])
 @pytest.mark.parametrize("nrhs", [4, 33])
 def test_subnormal_distances_between_far_boxes(form, nrhs):
     x = _points()
@@ -56,7 +56,7 @@ def test_subnormal_distances_between_far_boxes(form, nrhs):
         f = b.merged()
         lo = 700
     else:
-        f = SkelFMM(x, "laplace2d", 1e-6, 64, nrhs_max=nrhs, store_tiles=1 if form == "stored" else 0)
+        f = SkelFMM(x, "laplace2d", 1e-6, 64, nrhs_max=nrhs, store_tiles={"stored": 1, "symmetric": 2}.get(form, 0))
     q = torch.from_numpy(np.random.default_rng(93).uniform(0.5, 1.5, (lo + n, nrhs))).cuda().float()
     if lo:
         u, ref = torch.empty((nrhs, lo + n), device="cuda"), torch.empty((nrhs, lo + n), device="cuda", dtype=torch.float64)

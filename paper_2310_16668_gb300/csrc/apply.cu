@@ -360,11 +360,16 @@ constexpr bool ud_few(int nrhs) {
     return nrhs <= (sizeof(S) <= 8 ? kUnMaxRhs : 4);
 }
 // the default: a warp per stream (W = 8), unless the level has as many work
-// entries as such CTAs run at a time and short sums. 4 right-hand sides, W = 8
-// against W = 1: 1,016 entries of up to 61 inner indices 10.4, 14.5 us; 1,024 of
-// 56 10.8, 8.3; 2,054 of 56 14.9, 12.4; 5,705 of 21 30.8, 14.9; 1,504 of 129 14.9,
-// 20.6; 384 of 797 14.5, 39.4
-inline int ud_few_default(int ninner, int64_t work) { return kUdFew + (ninner <= 128 && work >= 1024 ? 1 : kUnWarps); }
+// entries as such CTAs run at a time and short sums (upward, where a warp has no
+// u_S += uhat to do as well, already at half of that for sums of two chunks). 4
+// right-hand sides, W = 8 against W = 1: down, 1,016 entries of up to 61 inner
+// indices 10.4, 14.5 us, 2,054 of 56 14.9, 12.4, 5,705 of 21 30.8, 14.9, 1,504 of 129
+// 14.9, 20.6; up, 392 of 55 6.2, 6.2, 603 of 56 8.1, 6.2, 1,022 of 57 10.1, 6.2, 384
+// of 797 14.5, 39.4
+inline int ud_few_default(bool down, int ninner, int64_t work) {
+    const bool by_warp = ninner <= 128 && work >= (!down && ninner <= 64 ? 512 : 1024);
+    return kUdFew + (by_warp ? 1 : kUnWarps);
+}
 
 // one level of the upward or downward pass; shape = 0: the level's setting
 // (autotuned for FP32, else the default rule)
@@ -385,7 +390,7 @@ void up_down(bool down, const DevicePlan* dp, int l, const S* T, S* X, int nrhs,
     }
     if (W == 0) {
         const std::vector<int64_t>& work = dp->ud_work_ptr[down ? 1 : 0][0];
-        W = few ? ud_few_default(ninner, work[l + 1] - work[l]) : ud_default_warps((ninner + kGT - 1) / kGT);
+        W = few ? ud_few_default(down, ninner, work[l + 1] - work[l]) : ud_default_warps((ninner + kGT - 1) / kGT);
     }
     if (W > kUdFew) {
         down ? ud_few_launch<S, true>(dp, l, W - kUdFew, nrhs, T, X, conj_op, st)
@@ -1479,7 +1484,7 @@ TuneReport device_autotune(DevicePlan* dp, int nrhs, bool allow_store, void* str
                 const float* T = (const float*)(down ? b->Tt : b->T);
                 const int ninner = down ? dp->up_level_maxk[l] : dp->up_level_maxr[l];
                 const std::vector<int64_t>& work = dp->ud_work_ptr[down][0];
-                const int def = few ? ud_few_default(ninner, work[l + 1] - work[l])
+                const int def = few ? ud_few_default(down != 0, ninner, work[l + 1] - work[l])
                                     : ud_default_warps((ninner + kGT - 1) / kGT);
                 double best_ms = 1e30, def_ms = 0;
                 int best = def;

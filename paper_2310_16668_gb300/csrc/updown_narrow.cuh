@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(32 * kUnWarps) updown_narrow_kernel(const UpBo
             next = entry_of(ch + 2 * kUnWarps);
 #pragma unroll
             for (int g0 = 0; g0 < 32; g0 += G) {
-                load_t(g0 + G < 32 ? 32 * ch + g0 + G : 32 * (ch + kUnWarps), b);
+                if (g0 >= jn) break;                         // (a short chunk is the last one)
+                if (jn == 32 || g0 + G < jn) load_t(g0 + G < 32 ? 32 * ch + g0 + G : 32 * (ch + kUnWarps), b);
 #pragma unroll
                 for (int q = 0; q < G; ++q)
                     if (g0 + q < jn) {
